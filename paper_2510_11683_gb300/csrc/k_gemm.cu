@@ -511,16 +511,52 @@ __device__ __forceinline__ void epi_dx(const GemmParams& p, const CUtensorMap* m
   }
 }
 
+// The dW GEMM reads and writes 8 bytes of dW per element whatever its K is; up
+// to about 2,000 rows that read-modify-write, not the tensor pipe, bounds it. A
+// reduce-add that misses L2 streams dW at 5.0 TB/s, one that finds its lines
+// there at up to 6.7 (plain copy: 6.4), so each warp fetches the lines of the
+// pair's next tile into L2 while it adds the current one, in halves (512-byte
+// row segments): whole tiles at once measured 5-12% slower, quarters and eighths
+// slower than no prefetch. Before -> after, in us: V 126464, H 4096: 829 -> 618
+// (31 rows), 835 -> 700 (505), 911 -> 844 (1012), 1204 -> 1045 (1521), 1470 ->
+// 1335 (2027); V 152064, H 3584: 855 -> 653 (62), 967 -> 907 (1012); V 32000,
+// H 2048: 106 -> 90 (62), 131 -> 121 (1012). From 2,500 rows on the two are within
+// the noise (1591 -> 1657, 1636 -> 1616 at 2536; 2489 -> 2568 at 4056). A dW
+// that L2 holds needs no fetching (V 8192, H 1024: 14 -> 18 at 62 rows), and row
+// segments that do not start on a 128-byte line gain nothing (V 50001, H 1032:
+// 86 -> 90 at 505 rows, 106 -> 102 at 1012).
+constexpr int64_t kDwPrefetchKb = 32;                      // K blocks: 2,048 rows
+constexpr int64_t kDwPrefetchMinBytes = int64_t(1) << 27;  // about L2's size
+
+__device__ __forceinline__ bool dw_prefetches(const GemmParams& p, const Work& w) {
+  return w.kb_total - w.kb_first <= kDwPrefetchKb && p.g.H % 32 == 0 &&
+         4 * (p.v_end - p.v_begin) * p.g.H >= kDwPrefetchMinBytes;
+}
+
+// Fetches half `part` (kBN / 2 columns, one 512-byte row segment per lane) of
+// this warp's 32 dW rows of tile t into L2 (columns past H and rows past V are
+// not touched).
+__device__ __forceinline__ void prefetch_dw(const GemmParams& p, const Unit& t, uint32_t rank,
+                                            int quarter, int lane, int part) {
+  const int64_t v = p.v_begin + (int64_t)t.m_blk * kPairM + (int64_t)rank * kBM + quarter * 32 + lane;
+  const int32_t h0 = t.n_blk * kBN + part * (kBN / 2);
+  if (v < p.g.V && h0 < p.g.H)
+    bulk_prefetch_l2(p.dW + v * p.g.H + h0, (uint32_t)min(kBN / 2, (int32_t)p.g.H - h0) * 4u);
+}
+
 // GEMM_DW: dW[v, h] += acc through TMA reduce-add of 32 x 32 fp32 sub-tiles
 // (the read-modify-write happens at L2; vocabulary rows >= V are clipped).
-// Accumulator row r is vocabulary entry v_begin + r.
+// Accumulator row r is vocabulary entry v_begin + r. `ahead`: the dW lines of
+// this pair's next tile `tn` are fetched into L2 meanwhile, half a tile at a time.
 __device__ __forceinline__ void epi_dw(const GemmParams& p, const CUtensorMap* map_c, const Unit& t,
-                                       int64_t row0, int lane, uint32_t tb, EpiStage& st) {
+                                       int64_t row0, int lane, uint32_t tb, EpiStage& st,
+                                       bool ahead, const Unit& tn, uint32_t rank, int quarter) {
   const int32_t h0 = t.n_blk * kBN;
   const int64_t v = p.v_begin + row0;
   if (v >= p.g.V) return;  // this warp's rows all lie past the vocabulary (warp-uniform)
 #pragma unroll 1
   for (int c = 0; c < kBN / 32; ++c) {
+    if (ahead && c % 4 == 0) prefetch_dw(p, tn, rank, quarter, lane, c / 4);
     if (h0 + c * 32 >= p.g.H) break;  // warp-uniform
     uint32_t raw[32];
     tmem_ld_32x32b_x32(tb + c * 32, raw);
@@ -732,6 +768,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     st.buf = 0;
     int it = 0;
     bool ok = true;
+    const bool ahead = KIND == GEMM_DW && dw_prefetches(p, wk);
+    if (ahead) {
+      const Unit t0 = unit_of<KIND>(wk, pair);
+      prefetch_dw(p, t0, rank, quarter, lane, 0);
+      prefetch_dw(p, t0, rank, quarter, lane, 1);
+    }
     for (int64_t u = pair; u < wk.units; u += num_pairs, ++it) {
       const Unit t = unit_of<KIND>(wk, u);
       const int acc = it % kBufs;
@@ -747,8 +789,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 #pragma unroll 1
         for (int g = 0; g < kNacc; ++g)
           epi_dx(p, &map_c, M, wk, t, t.n_blk * kNacc + g, row0, lane, tb + (uint32_t)(g * kBN), st);
+      } else {
+        const bool more = ahead && u + num_pairs < wk.units;
+        epi_dw(p, &map_c, t, row0, lane, tb, st, more, unit_of<KIND>(wk, more ? u + num_pairs : u),
+               rank, quarter);
       }
-      else epi_dw(p, &map_c, t, row0, lane, tb, st);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_addr(&tempty[acc]), 0));
