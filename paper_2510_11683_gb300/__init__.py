@@ -22,9 +22,15 @@ FLAG_KEEP_LOGITS = 1   # BGPO_FLAG_KEEP_LOGITS
 FLAG_PAIR_DW = 2       # BGPO_FLAG_PAIR_DW
 
 
+_TORCH = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _TORCH
+    if _TORCH is None:
+        import torch
+        _TORCH = torch
+    return _TORCH
 
 
 def problem(B, P, R, H, V, n_t, G, t_mode=T_IID, seed=0, loss_scale=None, trace=None,
@@ -87,9 +93,22 @@ def alloc_workspace(prob, device="cuda"):
     return ws
 
 
-def _ptr(t, dtype=None, name="tensor"):
+def _ptr(t, dtype=None, name="tensor", cur=None):
+    """Address of a contiguous CUDA tensor of `dtype` on the current device (None for None).
+
+    `cur`: the current device's index where the caller has it (_current_device)."""
     if t is None:
         return None
+    if cur is None:
+        cur = _current_device()      # also imports torch
+    if (isinstance(t, _TORCH.Tensor) and t.is_cuda and t.get_device() == cur
+            and (dtype is None or t.dtype is dtype) and t.is_contiguous()):
+        return t.data_ptr()
+    _refuse(t, dtype, name)
+
+
+def _refuse(t, dtype, name):
+    """Raises what is wrong with a tensor that _ptr does not take."""
     torch = _torch()
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
@@ -102,97 +121,112 @@ def _ptr(t, dtype=None, name="tensor"):
         raise ValueError(f"{name} is on {t.device}, but the current CUDA device is cuda:{cur}")
     if dtype is not None and t.dtype != dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
-    if not t.is_contiguous():
-        raise ValueError(f"{name} must be contiguous")
-    return t.data_ptr()
+    raise ValueError(f"{name} must be contiguous")
 
 
-def _stream(stream):
+def _current_device():
+    """Index of the current CUDA device, or -1 while CUDA is not initialised (no tensor
+    is on the GPU then, and _ptr refuses every tensor)."""
     torch = _torch()
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream
+    return torch._C._cuda_getDevice() if torch.cuda.is_initialized() else -1
+
+
+def _stream(stream, cur=None):
+    """Raw handle of `stream`, or of the current stream. torch.cuda.current_stream()
+    builds a Stream object for it (3.0 us); the handle alone takes 0.1 us."""
+    if stream is not None:
+        return stream.cuda_stream
+    torch = _torch()
+    if cur is None or cur < 0:
+        cur = torch.cuda.current_device()
+    return torch._C._cuda_getCurrentRawStream(cur)
 
 
 def sample_mask(prob, j, ws, t_out=None, mask_out=None, stream=None):
-    torch = _torch()
+    torch, cur = _torch(), _current_device()
     st = _lib.lib().bgpo_sample_mask(
-        ctypes.byref(prob), j, _ptr(ws, torch.uint8, "ws"), ws.numel(),
-        _ptr(t_out, torch.float32, "t_out"), _ptr(mask_out, torch.uint8, "mask_out"),
-        _stream(stream))
+        ctypes.byref(prob), j, _ptr(ws, torch.uint8, "ws", cur), ws.numel(),
+        _ptr(t_out, torch.float32, "t_out", cur), _ptr(mask_out, torch.uint8, "mask_out", cur),
+        _stream(stream, cur))
     _lib.check("bgpo_sample_mask", st)
 
 
 def elbo_fwd(prob, j, X, W, Y, ws, ell_out, stream=None):
-    torch = _torch()
+    torch, cur = _torch(), _current_device()
     st = _lib.lib().bgpo_elbo_fwd(
-        ctypes.byref(prob), j, _ptr(X, torch.bfloat16, "X"), _ptr(W, torch.bfloat16, "W"),
-        _ptr(Y, torch.int32, "Y"), _ptr(ws, torch.uint8, "ws"), ws.numel(),
-        _ptr(ell_out, torch.float32, "ell_out"), _stream(stream))
+        ctypes.byref(prob), j, _ptr(X, torch.bfloat16, "X", cur),
+        _ptr(W, torch.bfloat16, "W", cur), _ptr(Y, torch.int32, "Y", cur),
+        _ptr(ws, torch.uint8, "ws", cur), ws.numel(),
+        _ptr(ell_out, torch.float32, "ell_out", cur), _stream(stream, cur))
     _lib.check("bgpo_elbo_fwd", st)
 
 
 def bound_coeffs(prob, j, ell, ell_old, A, coef_out, g_out, ws, stream=None):
-    torch = _torch()
+    torch, cur = _torch(), _current_device()
     f32 = torch.float32
     st = _lib.lib().bgpo_bound_coeffs(
-        ctypes.byref(prob), j, _ptr(ell, f32, "ell"), _ptr(ell_old, f32, "ell_old"),
-        _ptr(A, f32, "A"), _ptr(coef_out, f32, "coef_out"), _ptr(g_out, f32, "g_out"),
-        _ptr(ws, torch.uint8, "ws"), ws.numel(), _stream(stream))
+        ctypes.byref(prob), j, _ptr(ell, f32, "ell", cur), _ptr(ell_old, f32, "ell_old", cur),
+        _ptr(A, f32, "A", cur), _ptr(coef_out, f32, "coef_out", cur),
+        _ptr(g_out, f32, "g_out", cur), _ptr(ws, torch.uint8, "ws", cur), ws.numel(),
+        _stream(stream, cur))
     _lib.check("bgpo_bound_coeffs", st)
 
 
 def vrpo_coeffs(prob, ell, ell_old, A, coef_out, R_out, ws, stream=None):
     """Eq. 7 coefficients from all n_t samples' l ([n_t, B] tensors)."""
-    torch = _torch()
+    torch, cur = _torch(), _current_device()
     f32 = torch.float32
     st = _lib.lib().bgpo_vrpo_coeffs(
-        ctypes.byref(prob), _ptr(ell, f32, "ell"), _ptr(ell_old, f32, "ell_old"),
-        _ptr(A, f32, "A"), _ptr(coef_out, f32, "coef_out"), _ptr(R_out, f32, "R_out"),
-        _ptr(ws, torch.uint8, "ws"), ws.numel(), _stream(stream))
+        ctypes.byref(prob), _ptr(ell, f32, "ell", cur), _ptr(ell_old, f32, "ell_old", cur),
+        _ptr(A, f32, "A", cur), _ptr(coef_out, f32, "coef_out", cur),
+        _ptr(R_out, f32, "R_out", cur), _ptr(ws, torch.uint8, "ws", cur), ws.numel(),
+        _stream(stream, cur))
     _lib.check("bgpo_vrpo_coeffs", st)
 
 
 def elbo_bwd_accumulate(prob, j, X, W, Y, coef, ws, dX, dW, stream=None):
-    torch = _torch()
+    torch, cur = _torch(), _current_device()
     f32 = torch.float32
     st = _lib.lib().bgpo_elbo_bwd_accumulate(
-        ctypes.byref(prob), j, _ptr(X, torch.bfloat16, "X"), _ptr(W, torch.bfloat16, "W"),
-        _ptr(Y, torch.int32, "Y"), _ptr(coef, f32, "coef"), _ptr(ws, torch.uint8, "ws"),
-        ws.numel(), _ptr(dX, f32, "dX"), _ptr(dW, f32, "dW"), _stream(stream))
+        ctypes.byref(prob), j, _ptr(X, torch.bfloat16, "X", cur),
+        _ptr(W, torch.bfloat16, "W", cur), _ptr(Y, torch.int32, "Y", cur),
+        _ptr(coef, f32, "coef", cur), _ptr(ws, torch.uint8, "ws", cur), ws.numel(),
+        _ptr(dX, f32, "dX", cur), _ptr(dW, f32, "dW", cur), _stream(stream, cur))
     _lib.check("bgpo_elbo_bwd_accumulate", st)
 
 
 def group_advantage(prob, rewards, A_out, stream=None):
-    torch = _torch()
+    torch, cur = _torch(), _current_device()
     st = _lib.lib().bgpo_group_advantage(
-        ctypes.byref(prob), _ptr(rewards, torch.float32, "rewards"),
-        _ptr(A_out, torch.float32, "A_out"), _stream(stream))
+        ctypes.byref(prob), _ptr(rewards, torch.float32, "rewards", cur),
+        _ptr(A_out, torch.float32, "A_out", cur), _stream(stream, cur))
     _lib.check("bgpo_group_advantage", st)
 
 
 def get_device_error(ws, stream=None):
     """(status, where) of the workspace's device error word (synchronises)."""
-    torch = _torch()
+    torch, cur = _torch(), _current_device()
     code = ctypes.c_int32(0)
     where = ctypes.c_int32(0)
-    st = _lib.lib().bgpo_get_device_error(_ptr(ws, torch.uint8, "ws"), ws.numel(),
-                                          ctypes.byref(code), ctypes.byref(where), _stream(stream))
+    st = _lib.lib().bgpo_get_device_error(_ptr(ws, torch.uint8, "ws", cur), ws.numel(),
+                                          ctypes.byref(code), ctypes.byref(where),
+                                          _stream(stream, cur))
     _lib.check("bgpo_get_device_error", st)
     return code.value, where.value
 
 
 def clear_device_error(ws, stream=None):
-    torch = _torch()
-    st = _lib.lib().bgpo_clear_device_error(_ptr(ws, torch.uint8, "ws"), ws.numel(),
-                                            _stream(stream))
+    torch, cur = _torch(), _current_device()
+    st = _lib.lib().bgpo_clear_device_error(_ptr(ws, torch.uint8, "ws", cur), ws.numel(),
+                                            _stream(stream, cur))
     _lib.check("bgpo_clear_device_error", st)
 
 
 def selftest_bounded_wait(ws, timeout_us=2000, stream=None):
     """Launches the bounded-wait self-test; read the result with get_device_error."""
-    torch = _torch()
-    st = _lib.lib().bgpo_selftest_bounded_wait(_ptr(ws, torch.uint8, "ws"), ws.numel(),
-                                               timeout_us, _stream(stream))
+    torch, cur = _torch(), _current_device()
+    st = _lib.lib().bgpo_selftest_bounded_wait(_ptr(ws, torch.uint8, "ws", cur), ws.numel(),
+                                               timeout_us, _stream(stream, cur))
     _lib.check("bgpo_selftest_bounded_wait", st)
 
 

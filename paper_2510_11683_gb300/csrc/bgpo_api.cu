@@ -10,6 +10,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <atomic>
 #include <mutex>
 
 #include "bgpo.h"
@@ -96,20 +97,30 @@ bgpo_status check_ws(const bgpo_problem* p, const void* ws, size_t ws_bytes, WsL
   return BGPO_OK;
 }
 
+// SM count of the current device, which must be a GB300. A device's attributes
+// do not change while the process lives, so each is asked for once.
+constexpr int kMaxDevices = 64;
+std::atomic<int> g_sms[kMaxDevices];   // 0: not asked yet, -1: not sm_103
+
 bgpo_status device_sms(int* num_sms) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) {
     cudaGetLastError();
     return BGPO_ERR_UNSUPPORTED_DEVICE;
   }
-  int major = 0, minor = 0, sms = 0;
-  if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    cudaGetLastError();
-    return BGPO_ERR_CUDA;
+  int sms = dev < kMaxDevices ? g_sms[dev].load(std::memory_order_relaxed) : 0;
+  if (sms == 0) {
+    int major = 0, minor = 0;
+    if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+      cudaGetLastError();
+      return BGPO_ERR_CUDA;
+    }
+    if (major != 10 || minor != 3) sms = -1;
+    if (dev < kMaxDevices) g_sms[dev].store(sms, std::memory_order_relaxed);
   }
-  if (major != 10 || minor != 3) return BGPO_ERR_UNSUPPORTED_DEVICE;
+  if (sms < 0) return BGPO_ERR_UNSUPPORTED_DEVICE;
   *num_sms = sms;
   return BGPO_OK;
 }
@@ -337,14 +348,15 @@ bgpo_status bgpo_elbo_bwd_accumulate(const bgpo_problem* prob, int32_t j, const 
   CUtensorMap map_xm_k, map_w_k, map_dz_k, map_w_mn, map_dz_mn, map_xmT_k;
   CUtensorMap map_dz_st, map_dxp_st, map_dw_red;
   const uint64_t dxp_rows = (uint64_t)dxp_row_block_cap(g) * kPairM;
-  if (!map_2d(&map_xm_k, w.xm, g.H, g.m_pad, g.H * 2, kBK, kBM) ||
-      !map_2d(&map_w_k, W, g.H, g.V, g.H * 2, kBK, kBNHalf) ||
+  // the recomputing dZ GEMM's maps (not needed with kept logits)
+  if ((!keep && (!map_2d(&map_xm_k, w.xm, g.H, g.m_pad, g.H * 2, kBK, kBM) ||
+                 !map_2d(&map_w_k, W, g.H, g.V, g.H * 2, kBK, kBNHalf) ||
+                 // epilogue destinations: 32-row sub-tiles of 128 bytes
+                 !map_2d(&map_dz_st, w.dz, zc, zr, zc * 2, 64, 32))) ||
       !map_2d(&map_dz_k, w.dz, zc, zr, zc * 2, kBK, kBM) ||
       !map_2d(&map_w_mn, W, g.H, g.V, g.H * 2, 64, kBK) ||
       !map_2d(&map_dz_mn, w.dz, zc, zr, zc * 2, 64, kBK) ||
       !map_2d(&map_xmT_k, w.xmT, zr, g.H, zr * 2, kBK, kBNHalf) ||
-      // epilogue destinations: 32-row sub-tiles of 128 bytes
-      !map_2d(&map_dz_st, w.dz, zc, zr, zc * 2, 64, 32) ||
       !map_2d(&map_dxp_st, w.dxp, g.H, dxp_rows, g.H * 4, 32, 32, CU_TENSOR_MAP_DATA_TYPE_FLOAT32) ||
       !map_2d(&map_dw_red, dW, g.H, g.V, g.H * 4, 32, 32, CU_TENSOR_MAP_DATA_TYPE_FLOAT32))
     return BGPO_ERR_CUDA;
