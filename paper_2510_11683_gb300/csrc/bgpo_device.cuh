@@ -314,6 +314,26 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint16_t cta_mask
       : "memory");
 }
 
+// ---- dependent launches --------------------------------------------------------------
+
+// Every kernel of the path is launched with programmatic stream serialization
+// (launch_dependent): its blocks may start while the kernel before it in the
+// stream still runs. pdl_wait() returns once that kernel has completed and its
+// writes are visible; nothing before it touches global memory other than the
+// kernel's own parameters. Each kernel waits in every block, so a kernel that
+// has completed implies that all kernels before it have.
+__device__ __forceinline__ void pdl_launch_dependents() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// The head of a kernel without a prologue of its own.
+__device__ __forceinline__ void pdl_begin() {
+  pdl_launch_dependents();
+  pdl_wait();
+}
+
 // ---- misc -----------------------------------------------------------------------
 
 __device__ __forceinline__ float warp_sum(float v) {

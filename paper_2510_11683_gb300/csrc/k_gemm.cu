@@ -619,30 +619,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int64_t num_pairs = gridDim.x >> 1;
   int32_t* err = p.w.err;
 
-  int32_t M = 0;
-  if (err[ERR_SAMPLE] == p.j) {
-    M = err[ERR_M];
-  } else if (blockIdx.x == 0 && threadIdx.x == 0) {
-    set_device_error(err, kStatusInvalidArg, kernel_id<KIND>() * 16 + 1);
-  }
-  if (!BGPO_IN_BOUNDS(err, M >= 0 && M <= p.g.m_cap, kernel_id<KIND>() * 16 + 9)) M = 0;
-  // first dZ / Xm^T row of this sample: nonzero only when it pairs with a
-  // pending sample (the masking set it; the forward does not use dZ)
-  const int64_t roff = KIND == GEMM_FWD ? 0 : row_offset(err[ERR_ROW_OFF], p.w.dz_rows, p.g.m_pad);
-  // dW: first K row, a multiple of kBK in [0, roff] (see ERR_DW_K0)
-  const int64_t k0 = KIND == GEMM_DW ? row_offset(err[ERR_DW_K0], roff + p.g.m_pad, p.g.m_pad) : 0;
-  const Work wk = make_work<KIND>(p, M, roff, k0);
-  if (KIND == GEMM_DW && blockIdx.x == 0 && threadIdx.x == 0) {
-    // a dW GEMM meant to complete a pair whose first sample is not pending
-    // adds this sample alone: the other sample's contribution is missing
-    if (p.pair_consume && err[ERR_PAIRED] != 1)
-      set_device_error(err, kStatusInvalidArg, kernel_id<KIND>() * 16 + 5);
-    err[ERR_PEND] = -1;  // nothing waits any more
-  }
-  // the split reduction after the dX GEMM reads the split count from here
-  if (KIND == GEMM_DX && blockIdx.x == 0 && threadIdx.x == 0) err[ERR_DX_SPLITS] = wk.splits;
-  if (pair >= wk.units) return;  // both CTAs of the pair, before any allocation
-
+  // the prologue touches no global memory: it runs while the kernel before this
+  // one finishes
   if (threadIdx.x == 0) {
     for (int s = 0; s < kSt; ++s) {
       mbar_init(smem_addr(&full[s]), 1);    // the even CTA's arrive.expect_tx
@@ -670,6 +648,32 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   cluster_sync();  // barriers of both CTAs initialised, TMEM allocated
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+
+  pdl_launch_dependents();
+  pdl_wait();
+
+  int32_t M = 0;
+  if (err[ERR_SAMPLE] == p.j) {
+    M = err[ERR_M];
+  } else if (blockIdx.x == 0 && threadIdx.x == 0) {
+    set_device_error(err, kStatusInvalidArg, kernel_id<KIND>() * 16 + 1);
+  }
+  if (!BGPO_IN_BOUNDS(err, M >= 0 && M <= p.g.m_cap, kernel_id<KIND>() * 16 + 9)) M = 0;
+  // first dZ / Xm^T row of this sample: nonzero only when it pairs with a
+  // pending sample (the masking set it; the forward does not use dZ)
+  const int64_t roff = KIND == GEMM_FWD ? 0 : row_offset(err[ERR_ROW_OFF], p.w.dz_rows, p.g.m_pad);
+  // dW: first K row, a multiple of kBK in [0, roff] (see ERR_DW_K0)
+  const int64_t k0 = KIND == GEMM_DW ? row_offset(err[ERR_DW_K0], roff + p.g.m_pad, p.g.m_pad) : 0;
+  const Work wk = make_work<KIND>(p, M, roff, k0);
+  if (KIND == GEMM_DW && blockIdx.x == 0 && threadIdx.x == 0) {
+    // a dW GEMM meant to complete a pair whose first sample is not pending
+    // adds this sample alone: the other sample's contribution is missing
+    if (p.pair_consume && err[ERR_PAIRED] != 1)
+      set_device_error(err, kStatusInvalidArg, kernel_id<KIND>() * 16 + 5);
+    err[ERR_PEND] = -1;  // nothing waits any more
+  }
+  // the split reduction after the dX GEMM reads the split count from here
+  if (KIND == GEMM_DX && blockIdx.x == 0 && threadIdx.x == 0) err[ERR_DX_SPLITS] = wk.splits;
 
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs) ----------------
@@ -768,7 +772,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     st.buf = 0;
     int it = 0;
     bool ok = true;
-    const bool ahead = KIND == GEMM_DW && dw_prefetches(p, wk);
+    const bool ahead = KIND == GEMM_DW && pair < wk.units && dw_prefetches(p, wk);
     if (ahead) {
       const Unit t0 = unit_of<KIND>(wk, pair);
       prefetch_dw(p, t0, rank, quarter, lane, 0);
@@ -822,8 +826,7 @@ cudaError_t launch_kind(const CUtensorMap& ma, const CUtensorMap& mb, const CUte
   cudaError_t e = cudaFuncSetAttribute(k_gemm<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
-  k_gemm<KIND><<<2 * p.num_pairs, kThreads, smem, s>>>(ma, mb, mc, p);
-  return cudaGetLastError();
+  return launch_dependent(k_gemm<KIND>, dim3(2 * p.num_pairs), kThreads, smem, s, ma, mb, mc, p);
 }
 
 }  // namespace

@@ -39,6 +39,7 @@ __device__ __forceinline__ int32_t rows_of_sample(int32_t* err, int32_t j, int32
 constexpr int kScanThreads = 1024;
 
 __global__ void __launch_bounds__(kScanThreads) k_mask_compact(MaskArgs a, WsPtrs w) {
+  pdl_begin();
   __shared__ int32_t warp_excl[32];
   __shared__ int32_t s_carry;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -156,8 +157,9 @@ __global__ void __launch_bounds__(kScanThreads) k_mask_compact(MaskArgs a, WsPtr
 // Rows [M, round_up(M, 256)) are zero-filled so that the GEMM pair tiles and
 // the K padding of the dW GEMM read zeros.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_gather(Geometry g, int32_t j, const uint4* __restrict__ X,
-                                                const int32_t* __restrict__ Y, WsPtrs w) {
+__global__ void __launch_bounds__(256) k_gather(Geometry g, int32_t j, const uint4* X, const int32_t* Y,
+                                                WsPtrs w) {
+  pdl_begin();
   const int32_t M = rows_of_sample(w.err, j, KID_GATHER);
   if (!BGPO_IN_BOUNDS(w.err, M <= g.m_cap, KID_GATHER * 16 + 9)) return;
   const int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -175,13 +177,13 @@ __global__ void __launch_bounds__(256) k_gather(Geometry g, int32_t j, const uin
       uint4 q[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k)
-        if (v0 + 32 * k < nvec) q[k] = __ldg(src + v0 + 32 * k);
+        if (v0 + 32 * k < nvec) q[k] = src[v0 + 32 * k];
 #pragma unroll
       for (int k = 0; k < 8; ++k)
         if (v0 + 32 * k < nvec) dst[v0 + 32 * k] = q[k];
     }
     if (lane == 0) {
-      const int32_t y = __ldg(Y + idx);
+      const int32_t y = Y[idx];
       (void)BGPO_IN_BOUNDS(w.err, y >= 0 && y < g.V, KID_GATHER * 16 + 11);  // a target outside V
       w.tgt[r] = y;
     }
@@ -208,6 +210,7 @@ constexpr int kLseBatch = 8;
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_lse_combine(Geometry g, int32_t j, bool kept_logits,
                                                      WsPtrs w) {
+  pdl_begin();
   const int32_t M = rows_of_sample(w.err, j, KID_LSE_COMBINE);
   if (blockIdx.x == 0 && threadIdx.x == 0)
     w.err[ERR_LOGITS] = (kept_logits && w.err[ERR_SAMPLE] == j) ? 1 : 0;
@@ -261,8 +264,8 @@ constexpr int kDzVec = 4;                           // 8-column vectors per thre
 constexpr int kDzItemVecs = kDzThreads * kDzVec;    // 1024 vectors = 8192 columns
 
 __global__ void __launch_bounds__(kDzThreads, 4)
-    k_dz_from_logits(Geometry g, int32_t j, int64_t chunk, const float* __restrict__ coef,
-                     WsPtrs w) {
+    k_dz_from_logits(Geometry g, int32_t j, int64_t chunk, const float* coef, WsPtrs w) {
+  pdl_begin();
   const int32_t M = rows_of_sample(w.err, j, KID_DZ_FROM_LOGITS);
   if (w.err[ERR_LOGITS] != 1) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -280,11 +283,11 @@ __global__ void __launch_bounds__(kDzThreads, 4)
   const int64_t dvec = w.dz_cols / 8;
   const int64_t per_row = ceil_div(nvec, kDzItemVecs);
   const int64_t items = round_up(M, kPairM) * per_row;
-  const float4* __restrict__ zc = reinterpret_cast<const float4*>(w.zc) + v_begin / 4;
+  const float4* zc = reinterpret_cast<const float4*>(w.zc) + v_begin / 4;
   // this sample's dZ rows start at the pairing offset (0 without pairing)
-  uint4* __restrict__ dz = reinterpret_cast<uint4*>(w.dz) +
-                           row_offset(w.err[ERR_ROW_OFF], w.dz_rows, g.m_pad) * dvec +
-                           (w.dz_chunk_local ? 0 : v_begin / 8);
+  uint4* dz = reinterpret_cast<uint4*>(w.dz) +
+              row_offset(w.err[ERR_ROW_OFF], w.dz_rows, g.m_pad) * dvec +
+              (w.dz_chunk_local ? 0 : v_begin / 8);
   const int32_t V = (int32_t)g.V;
   for (int64_t q = blockIdx.x; q < items; q += gridDim.x) {
     const int64_t r = q / per_row;
@@ -342,6 +345,7 @@ __global__ void __launch_bounds__(kDzThreads, 4)
 // per sequence, lane-strided sums then a fixed xor tree (deterministic).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_seq_reduce(Geometry g, int32_t j, WsPtrs w, float* ell_out) {
+  pdl_begin();
   const int32_t M = rows_of_sample(w.err, j, KID_SEQ_REDUCE);
   const int64_t b = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -361,9 +365,10 @@ __global__ void __launch_bounds__(256) k_seq_reduce(Geometry g, int32_t j, WsPtr
 //   d = l - l_old; A >= 0: g = (1 + d) A / n_t, dg/dl = A / n_t (Lemma 1)
 //                  A <  0: g = e^d A / n_t,    dg/dl = e^d A / n_t (Lemma 2)
 // ---------------------------------------------------------------------------
-__global__ void k_bound_coeffs(int32_t B, int32_t n_t, float loss_scale, const float* __restrict__ ell,
-                               const float* __restrict__ ell_old, const float* __restrict__ A,
-                               float* coef_out, float* g_out, int32_t* err) {
+__global__ void k_bound_coeffs(int32_t B, int32_t n_t, float loss_scale, const float* ell,
+                               const float* ell_old, const float* A, float* coef_out, float* g_out,
+                               int32_t* err) {
+  pdl_begin();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
   const float d = ell[b] - ell_old[b];
@@ -382,9 +387,10 @@ __global__ void k_bound_coeffs(int32_t B, int32_t n_t, float loss_scale, const f
 // VRPO (Eq. 7): R_hat = e^{mean_j (l - l_old)} A and dL/dl_{b,j} =
 // -loss_scale A e^{mean_j d} / n_t for every j (Sec. 3.2). l, l_old [n_t, B].
 // ---------------------------------------------------------------------------
-__global__ void k_vrpo_coeffs(int32_t B, int32_t n_t, float loss_scale, const float* __restrict__ ell,
-                              const float* __restrict__ ell_old, const float* __restrict__ A,
-                              float* coef_out, float* R_out, int32_t* err) {
+__global__ void k_vrpo_coeffs(int32_t B, int32_t n_t, float loss_scale, const float* ell,
+                              const float* ell_old, const float* A, float* coef_out, float* R_out,
+                              int32_t* err) {
+  pdl_begin();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
   float sum_d = 0.f;
@@ -410,7 +416,8 @@ constexpr int kDxrThreads = 256;
 constexpr int kDxrVec = 4;
 
 __global__ void __launch_bounds__(kDxrThreads) k_dx_reduce(Geometry g, int32_t j, WsPtrs w,
-                                                           float* __restrict__ dX) {
+                                                           float* dX) {
+  pdl_begin();
   const int32_t M = rows_of_sample(w.err, j, KID_DX_REDUCE);
   const int64_t r = blockIdx.x;
   if (r >= M) return;
@@ -424,7 +431,7 @@ __global__ void __launch_bounds__(kDxrThreads) k_dx_reduce(Geometry g, int32_t j
   const int64_t split_stride = mb * kPairM * g.H / 4;
   const int32_t idx = w.rows[r];
   if (!BGPO_IN_BOUNDS(w.err, idx >= 0 && idx < g.m_cap, KID_DX_REDUCE * 16 + 9)) return;
-  const float4* __restrict__ src = reinterpret_cast<const float4*>(w.dxp) + r * (g.H / 4);
+  const float4* src = reinterpret_cast<const float4*>(w.dxp) + r * (g.H / 4);
   float4* dst = reinterpret_cast<float4*>(dX) + (int64_t)idx * (g.H / 4);
   const int64_t nvec = g.H / 4;
   for (int64_t h0 = threadIdx.x; h0 < nvec; h0 += (int64_t)kDxrThreads * kDxrVec) {
@@ -478,6 +485,7 @@ constexpr int kTrChunks = kTrRows * kTrCols / 8 / kTrThreads;   // 16-byte chunk
 
 __global__ void __launch_bounds__(kTrThreads) k_xm_transpose(Geometry g, int32_t j, bool defer,
                                                              WsPtrs w) {
+  pdl_begin();
   const int32_t M = rows_of_sample(w.err, j, KID_XM_TRANSPOSE);
   if (!BGPO_IN_BOUNDS(w.err, M <= g.m_cap, KID_XM_TRANSPOSE * 16 + 9)) return;
   const int64_t off = row_offset(w.err[ERR_ROW_OFF], w.dz_rows, g.m_pad);
@@ -496,8 +504,8 @@ __global__ void __launch_bounds__(kTrThreads) k_xm_transpose(Geometry g, int32_t
   const int64_t h0 = (int64_t)blockIdx.y * kTrCols;
   if (r0 >= round_up(M, kPairM)) return;  // block-uniform
   __shared__ __align__(16) uint16_t tile[kTrRows * kTrPitch];
-  const uint16_t* __restrict__ xm = static_cast<const uint16_t*>(w.xm);
-  uint16_t* __restrict__ xmT = static_cast<uint16_t*>(w.xmT);
+  const uint16_t* xm = static_cast<const uint16_t*>(w.xm);
+  uint16_t* xmT = static_cast<uint16_t*>(w.xmT);
   uint4 v[kTrChunks];
 #pragma unroll
   for (int i = 0; i < kTrChunks; ++i) {   // chunk c: row c / 8, columns (c % 8) * 8 ..
@@ -535,7 +543,8 @@ __global__ void __launch_bounds__(kTrThreads) k_xm_transpose(Geometry g, int32_t
 // ---------------------------------------------------------------------------
 // Eq. 18 over consecutive groups of G rewards (population std; 0 if std = 0).
 // ---------------------------------------------------------------------------
-__global__ void k_group_advantage(int32_t B, int32_t G, const float* __restrict__ r, float* A) {
+__global__ void k_group_advantage(int32_t B, int32_t G, const float* r, float* A) {
+  pdl_begin();
   const int64_t grp = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (grp * G >= B) return;
   const float* x = r + grp * G;
@@ -554,6 +563,7 @@ __global__ void k_group_advantage(int32_t B, int32_t G, const float* __restrict_
 // record BGPO_ERR_TIMEOUT in the error word.
 // ---------------------------------------------------------------------------
 __global__ void k_selftest_wait(int32_t* err, uint64_t timeout_ns) {
+  pdl_begin();
   __shared__ __align__(8) uint64_t bar;
   __shared__ int abort_flag;
   const uint32_t b = smem_addr(&bar);
@@ -571,8 +581,7 @@ __global__ void k_selftest_wait(int32_t* err, uint64_t timeout_ns) {
 }  // namespace
 
 cudaError_t launch_selftest_wait(int32_t* err, uint64_t timeout_ns, cudaStream_t s) {
-  k_selftest_wait<<<1, 32, 0, s>>>(err, timeout_ns);
-  return cudaGetLastError();
+  return launch_dependent(k_selftest_wait, 1, 32, 0, s, err, timeout_ns);
 }
 
 WsPtrs ws_pointers(void* ws, const WsLayout& L, bool forward_only) {
@@ -600,22 +609,19 @@ WsPtrs ws_pointers(void* ws, const WsLayout& L, bool forward_only) {
 }
 
 cudaError_t launch_mask_compact(const MaskArgs& a, const WsPtrs& w, cudaStream_t s) {
-  k_mask_compact<<<1, kScanThreads, 0, s>>>(a, w);
-  return cudaGetLastError();
+  return launch_dependent(k_mask_compact, 1, kScanThreads, 0, s, a, w);
 }
 
 cudaError_t launch_gather(const Geometry& g, int32_t j, const void* X, const int32_t* Y,
                           const WsPtrs& w, cudaStream_t s) {
   const unsigned grid = (unsigned)ceil_div(g.m_pad, 8);
-  k_gather<<<grid, 256, 0, s>>>(g, j, static_cast<const uint4*>(X), Y, w);
-  return cudaGetLastError();
+  return launch_dependent(k_gather, grid, 256, 0, s, g, j, static_cast<const uint4*>(X), Y, w);
 }
 
 cudaError_t launch_lse_combine(const Geometry& g, int32_t j, bool kept_logits, const WsPtrs& w,
                                cudaStream_t s) {
   const unsigned grid = (unsigned)ceil_div(g.m_cap, 8);
-  k_lse_combine<<<grid, 256, 0, s>>>(g, j, kept_logits, w);
-  return cudaGetLastError();
+  return launch_dependent(k_lse_combine, grid, 256, 0, s, g, j, kept_logits, w);
 }
 
 cudaError_t launch_dz_from_logits(const Geometry& g, int32_t j, int64_t chunk, const float* coef,
@@ -623,51 +629,46 @@ cudaError_t launch_dz_from_logits(const Geometry& g, int32_t j, int64_t chunk, c
   // 4 resident CTAs per SM; never more CTAs than the largest sample has items
   const int64_t most = g.m_pad * ceil_div(g.vc / 8, kDzItemVecs);
   const int64_t grid = most < 4 * (int64_t)num_sms ? most : 4 * (int64_t)num_sms;
-  k_dz_from_logits<<<(unsigned)grid, kDzThreads, 0, s>>>(g, j, chunk, coef, w);
-  return cudaGetLastError();
+  return launch_dependent(k_dz_from_logits, (unsigned)grid, kDzThreads, 0, s, g, j, chunk, coef,
+                          w);
 }
 
 cudaError_t launch_seq_reduce(const Geometry& g, int32_t j, const WsPtrs& w, float* ell_out,
                               cudaStream_t s) {
   const unsigned grid = (unsigned)ceil_div(g.B, 8);
-  k_seq_reduce<<<grid, 256, 0, s>>>(g, j, w, ell_out);
-  return cudaGetLastError();
+  return launch_dependent(k_seq_reduce, grid, 256, 0, s, g, j, w, ell_out);
 }
 
 cudaError_t launch_bound_coeffs(int32_t B, int32_t n_t, float loss_scale, const float* ell,
                                 const float* ell_old, const float* A, float* coef_out,
                                 float* g_out, const WsPtrs& w, cudaStream_t s) {
-  k_bound_coeffs<<<(unsigned)ceil_div(B, 256), 256, 0, s>>>(B, n_t, loss_scale, ell, ell_old, A,
-                                                            coef_out, g_out, w.err);
-  return cudaGetLastError();
+  return launch_dependent(k_bound_coeffs, (unsigned)ceil_div(B, 256), 256, 0, s, B, n_t, loss_scale,
+                          ell, ell_old, A, coef_out, g_out, w.err);
 }
 
 cudaError_t launch_vrpo_coeffs(int32_t B, int32_t n_t, float loss_scale, const float* ell,
                                const float* ell_old, const float* A, float* coef_out, float* R_out,
                                const WsPtrs& w, cudaStream_t s) {
-  k_vrpo_coeffs<<<(unsigned)ceil_div(B, 256), 256, 0, s>>>(B, n_t, loss_scale, ell, ell_old, A,
-                                                           coef_out, R_out, w.err);
-  return cudaGetLastError();
+  return launch_dependent(k_vrpo_coeffs, (unsigned)ceil_div(B, 256), 256, 0, s, B, n_t, loss_scale,
+                          ell, ell_old, A, coef_out, R_out, w.err);
 }
 
 cudaError_t launch_dx_reduce(const Geometry& g, int32_t j, const WsPtrs& w, float* dX,
                              cudaStream_t s) {
-  k_dx_reduce<<<(unsigned)g.m_cap, kDxrThreads, 0, s>>>(g, j, w, dX);
-  return cudaGetLastError();
+  return launch_dependent(k_dx_reduce, (unsigned)g.m_cap, kDxrThreads, 0, s, g, j, w, dX);
 }
 
 cudaError_t launch_xm_transpose(const Geometry& g, int32_t j, bool defer, const WsPtrs& w,
                                 cudaStream_t s) {
   const dim3 grid((unsigned)(g.m_pad / kTrRows), (unsigned)ceil_div(g.H, kTrCols));
-  k_xm_transpose<<<grid, kTrThreads, 0, s>>>(g, j, defer, w);
-  return cudaGetLastError();
+  return launch_dependent(k_xm_transpose, grid, kTrThreads, 0, s, g, j, defer, w);
 }
 
 cudaError_t launch_group_advantage(int32_t B, int32_t G, const float* rewards, float* A_out,
                                    cudaStream_t s) {
   const int64_t groups = B / G;
-  k_group_advantage<<<(unsigned)ceil_div(groups, 128), 128, 0, s>>>(B, G, rewards, A_out);
-  return cudaGetLastError();
+  return launch_dependent(k_group_advantage, (unsigned)ceil_div(groups, 128), 128, 0, s, B, G,
+                          rewards, A_out);
 }
 
 }  // namespace bgpo
