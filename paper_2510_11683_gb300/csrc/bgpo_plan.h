@@ -99,13 +99,21 @@ BGPO_HD int64_t xm_row_groups(int64_t tiles_m, int64_t H) {
 // `groups` row groups: group g holds row blocks [g tm / G, (g + 1) tm / G),
 // its units follow those of the groups before it, and consecutive units of a
 // group share a vocabulary tile.
+// (32-bit arithmetic: at most 2^14 row blocks times 2^16 vocabulary tiles)
 BGPO_HD void row_group_tile(int64_t u, int64_t tiles_m, int64_t tiles_n, int64_t groups,
                             int64_t* m_blk, int64_t* n_blk) {
-  int64_t g = 0;
-  while (g + 1 < groups && ((g + 1) * tiles_m / groups) * tiles_n <= u) ++g;
-  const int64_t r0 = g * tiles_m / groups;
-  const int64_t rows = (g + 1) * tiles_m / groups - r0;
-  const int64_t local = u - r0 * tiles_n;
+  const uint32_t tm = (uint32_t)tiles_m, tn = (uint32_t)tiles_n, ng = (uint32_t)groups;
+  uint32_t r0 = 0, rows = tm, local = (uint32_t)u;
+  if (ng > 1) {
+    uint32_t g = 0, end = tm / ng;   // end = (g + 1) tm / ng
+    while (g + 1 < ng && end * tn <= local) {
+      r0 = end;
+      ++g;
+      end = (g + 1) * tm / ng;
+    }
+    rows = end - r0;
+    local -= r0 * tn;
+  }
   *n_blk = local / rows;
   *m_blk = r0 + local % rows;
 }
@@ -115,23 +123,29 @@ BGPO_HD void row_group_tile(int64_t u, int64_t tiles_m, int64_t tiles_n, int64_t
 // wave-quantised time ceil(tiles*s/pairs)/s is within 8% of the ideal
 // tiles/pairs, else the best s. s * mb never exceeds `row_block_cap`, which
 // bounds the partial buffer independently of the SM count.
+// Integers only: every thread of the GEMM runs this, and 16 rounds of 64-bit and
+// double-precision divisions took 3 us of its start.
 BGPO_HD int dx_splits(int64_t mb, int64_t tiles_n, int num_pairs, int64_t k_blocks,
                       int64_t row_block_cap) {
-  const int64_t tiles_mn = mb * tiles_n;
-  const int num_sms = num_pairs;
-  if (tiles_mn <= 0 || num_sms <= 0) return 1;
-  int64_t smax = kMaxSplits;
-  if (k_blocks < smax) smax = k_blocks > 0 ? k_blocks : 1;
-  if (row_block_cap / mb < smax) smax = row_block_cap / mb > 0 ? row_block_cap / mb : 1;
-  const double ideal = (double)tiles_mn / (double)num_sms;
-  int best = 1;
-  double best_t = 1e300;
-  for (int s = 1; s <= smax; ++s) {
-    const double t = (double)ceil_div(tiles_mn * s, num_sms) / (double)s;
-    if (t <= ideal * 1.08) return s;
-    if (t < best_t) { best_t = t; best = s; }
+  if (mb * tiles_n <= 0 || num_pairs <= 0) return 1;
+  const uint32_t tiles = (uint32_t)(mb * tiles_n), pairs = (uint32_t)num_pairs;
+  uint32_t smax = kMaxSplits;
+  if (k_blocks < (int64_t)smax) smax = k_blocks > 0 ? (uint32_t)k_blocks : 1;
+  const uint32_t room = (uint32_t)row_block_cap / (uint32_t)mb;
+  if (room < smax) smax = room > 0 ? room : 1;
+  const uint32_t q = tiles / pairs, r = tiles % pairs;
+  uint32_t full = 0, rest = 0;       // tiles * s = full * pairs + rest
+  uint32_t best = 1, best_waves = 0;
+  for (uint32_t s = 1; s <= smax; ++s) {
+    full += q;
+    rest += r;
+    if (rest >= pairs) { rest -= pairs; ++full; }
+    const uint32_t waves = full + (rest ? 1u : 0u);
+    // waves / s <= 1.08 tiles / pairs
+    if ((uint64_t)waves * pairs * 25 <= (uint64_t)tiles * s * 27) return (int)s;
+    if (best_waves == 0 || waves * best < best_waves * s) { best = s; best_waves = waves; }
   }
-  return best;
+  return (int)best;
 }
 
 // Width of the backward's vocabulary chunks. `request` 0 asks for the

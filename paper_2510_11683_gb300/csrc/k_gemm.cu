@@ -69,11 +69,14 @@ struct GemmParams {
   bool pair_consume;
 };
 
+// (32 bits hold every count: at most 2^14 row blocks, 2^16 vocabulary tiles, 64
+// hidden-size tiles, 2^18 K blocks)
 struct Work {
-  int64_t units, tiles_m, tiles_n, kb_total;
-  int64_t kb_first;  // first K block (dW: a partner already added is skipped)
-  int64_t groups;    // forward and dZ: row groups (xm_row_groups)
-  int splits;
+  int32_t units, tiles_m, tiles_n, kb_total;
+  int32_t kb_first;  // first K block (dW: a partner already added is skipped)
+  int32_t groups;    // forward and dZ: row groups (xm_row_groups)
+  int32_t splits;
+  int32_t rows;      // A rows that hold data: CTAs and warps wholly past them skip theirs
 };
 
 struct Unit {
@@ -90,17 +93,18 @@ __device__ __forceinline__ Work make_work(const GemmParams& p, int32_t M, int64_
   w.splits = 1;
   w.kb_first = 0;
   w.groups = 1;
+  w.rows = M;
   if (KIND == GEMM_FWD || KIND == GEMM_DZ) {
-    w.tiles_m = ceil_div(M, kPairM);
-    w.tiles_n = KIND == GEMM_FWD ? p.g.n_vt : ceil_div(p.v_end - p.v_begin, kBN);
+    w.tiles_m = (int32_t)ceil_div(M, kPairM);
+    w.tiles_n = (int32_t)(KIND == GEMM_FWD ? p.g.n_vt : ceil_div(p.v_end - p.v_begin, kBN));
     // a last K block past H reads the tensor maps' zero fill
-    w.kb_total = ceil_div(p.g.H, kBK);
+    w.kb_total = (int32_t)ceil_div(p.g.H, kBK);
     w.units = w.tiles_m * w.tiles_n;
-    w.groups = xm_row_groups(w.tiles_m, p.g.H);
+    w.groups = (int32_t)xm_row_groups(w.tiles_m, p.g.H);
   } else if (KIND == GEMM_DX) {
-    w.tiles_m = ceil_div(M, kPairM);
-    w.tiles_n = dx_tiles_n(p.g.tiles_h);
-    w.kb_total = ceil_div(p.v_end - p.v_begin, kBK);
+    w.tiles_m = (int32_t)ceil_div(M, kPairM);
+    w.tiles_n = (int32_t)dx_tiles_n(p.g.tiles_h);
+    w.kb_total = (int32_t)ceil_div(p.v_end - p.v_begin, kBK);
     // one split count for every chunk of the sample (the partials of split s
     // accumulate over the chunks), bounded by the narrowest chunk's K blocks
     w.splits = w.tiles_m > 0 ? dx_splits(w.tiles_m, w.tiles_n, p.num_pairs, p.g.kb_vc_min,
@@ -108,17 +112,17 @@ __device__ __forceinline__ Work make_work(const GemmParams& p, int32_t M, int64_
                              : 1;
     w.units = w.tiles_m * w.tiles_n * w.splits;
   } else {  // GEMM_DW
-    w.tiles_m = ceil_div(p.v_end - p.v_begin, kPairM);
-    w.tiles_n = p.g.tiles_h;
-    w.kb_total = ceil_div(roff + M, kBK);
-    w.kb_first = k0 / kBK;
+    w.tiles_m = (int32_t)ceil_div(p.v_end - p.v_begin, kPairM);
+    w.tiles_n = (int32_t)p.g.tiles_h;
+    w.kb_total = (int32_t)ceil_div(roff + M, kBK);
+    w.kb_first = (int32_t)(k0 / kBK);
     w.units = w.kb_total > w.kb_first ? w.tiles_m * w.tiles_n : 0;
   }
   return w;
 }
 
 template <int KIND>
-__device__ __forceinline__ Unit unit_of(const Work& w, int64_t u) {
+__device__ __forceinline__ Unit unit_of(const Work& w, int32_t u) {
   Unit t;
   t.split = 0;
   if (KIND == GEMM_FWD || KIND == GEMM_DZ) {
@@ -129,25 +133,25 @@ __device__ __forceinline__ Unit unit_of(const Work& w, int64_t u) {
     t.m_blk = (int32_t)m;
     t.n_blk = (int32_t)n;
     t.kb0 = 0;
-    t.kb_n = (int32_t)w.kb_total;
+    t.kb_n = w.kb_total;
   } else if (KIND == GEMM_DX) {
     // consecutive units share a row block of dZ (measured 2% faster than
     // sharing a column block of W, and than grouped rasters)
-    const int64_t per_split = w.tiles_m * w.tiles_n;
-    t.split = (int32_t)(u / per_split);
-    const int64_t rem = u % per_split;
-    t.m_blk = (int32_t)(rem / w.tiles_n);
-    t.n_blk = (int32_t)(rem % w.tiles_n);
-    const int64_t k0 = (int64_t)t.split * w.kb_total / w.splits;
-    const int64_t k1 = (int64_t)(t.split + 1) * w.kb_total / w.splits;
+    const uint32_t per_split = (uint32_t)(w.tiles_m * w.tiles_n);
+    const uint32_t split = (uint32_t)u / per_split, rem = (uint32_t)u % per_split;
+    t.split = (int32_t)split;
+    t.m_blk = (int32_t)(rem / (uint32_t)w.tiles_n);
+    t.n_blk = (int32_t)(rem % (uint32_t)w.tiles_n);
+    const uint32_t k0 = split * (uint32_t)w.kb_total / (uint32_t)w.splits;
+    const uint32_t k1 = (split + 1) * (uint32_t)w.kb_total / (uint32_t)w.splits;
     t.kb0 = (int32_t)k0;
     t.kb_n = (int32_t)(k1 - k0);
   } else {
     // consecutive units share a vocabulary block of dZ^T
-    t.m_blk = (int32_t)(u / w.tiles_n);
-    t.n_blk = (int32_t)(u % w.tiles_n);
-    t.kb0 = (int32_t)w.kb_first;
-    t.kb_n = (int32_t)(w.kb_total - w.kb_first);
+    t.m_blk = (int32_t)((uint32_t)u / (uint32_t)w.tiles_n);
+    t.n_blk = (int32_t)((uint32_t)u % (uint32_t)w.tiles_n);
+    t.kb0 = w.kb_first;
+    t.kb_n = w.kb_total - w.kb_first;
   }
   return t;
 }
@@ -194,16 +198,27 @@ __device__ __forceinline__ int64_t b_base(const GemmParams& p) {
   return KIND == GEMM_DZ ? p.v_begin : 0;
 }
 
+// Whether this CTA's 128 rows of a K-major A tile hold any masked row. A tile
+// past them is not loaded: the MMA multiplies what the stage happens to hold,
+// into accumulator rows that no epilogue reads. With the epilogues' row checks
+// this leaves out up to three quarters of dZ's traffic at few rows: 4096 x 126464
+// head, one response of 99 and 221 masked rows, step 2087 -> 2004 us; 2048 x 32000
+// head, 301 to 424 rows, 1125 -> 1060 us (with the split rule in integers).
+__device__ __forceinline__ bool a_has_rows(const Work& w, const Unit& t, uint32_t rank) {
+  return t.m_blk * kPairM + (int32_t)rank * kBM < w.rows;
+}
+
 // Bytes this CTA's copies deliver for one stage of unit t (boxes that would lie
 // wholly outside the operand are not issued; their MMA outputs are discarded).
 template <int KIND>
-__device__ __forceinline__ uint32_t stage_bytes(const GemmParams& p, const Unit& t, uint32_t rank) {
+__device__ __forceinline__ uint32_t stage_bytes(const GemmParams& p, const Work& w, const Unit& t,
+                                                uint32_t rank) {
   const int64_t a0 = (int64_t)t.m_blk * kPairM + (int64_t)rank * kBM;
   const int64_t b0 =
       b_base<KIND>(p) + (int64_t)t.n_blk * Shape<KIND>::nacc * kBN + (int64_t)rank * kBNHalf;
   uint32_t bytes = 0;
   if (!Majors<KIND>::a_mn) {
-    bytes += kTileABytes;
+    if (a_has_rows(w, t, rank)) bytes += kTileABytes;
   } else {
     // dZ^T vocabulary columns of this CTA inside the dZ buffer
     for (int c = 0; c < kBM / 64; ++c)
@@ -224,17 +239,17 @@ __device__ __forceinline__ uint32_t stage_bytes(const GemmParams& p, const Unit&
 // `roff`; its K blocks count from the chunk's first vocabulary entry, which
 // lies at dZ column dz_col0 and W row v_begin.
 template <int KIND>
-__device__ __forceinline__ void load_stage(const GemmParams& p, const CUtensorMap* ma,
-                                           const CUtensorMap* mb, uint32_t sa, uint32_t sb,
-                                           uint32_t cbar, const Unit& t, int32_t kb,
-                                           uint32_t rank, int64_t roff) {
+__device__ __forceinline__ void load_stage(const GemmParams& p, const Work& w,
+                                           const CUtensorMap* ma, const CUtensorMap* mb,
+                                           uint32_t sa, uint32_t sb, uint32_t cbar, const Unit& t,
+                                           int32_t kb, uint32_t rank, int64_t roff) {
   const int32_t a0 =
       t.m_blk * kPairM + (int32_t)rank * kBM + (KIND == GEMM_DX ? (int32_t)roff : 0);
   const int64_t b0 =
       b_base<KIND>(p) + (int64_t)t.n_blk * Shape<KIND>::nacc * kBN + (int64_t)rank * kBNHalf;
   if (!Majors<KIND>::a_mn) {
     const int32_t ka = kb * kBK + (KIND == GEMM_DX ? (int32_t)p.dz_col0 : 0);
-    tma_load_2d_pair(sa, ma, cbar, ka, a0);
+    if (a_has_rows(w, t, rank)) tma_load_2d_pair(sa, ma, cbar, ka, a0);
   } else {
     // dZ^T rows of this CTA: 2 boxes of 64 vocabulary columns x 64 masked rows
 #pragma unroll
@@ -314,6 +329,7 @@ __device__ __forceinline__ void stage_row(uint32_t sbuf, int lane, const uint4 (
 __device__ __forceinline__ void epi_fwd(const GemmParams& p, const CUtensorMap* map_c, int32_t M,
                                         const Unit& t, int64_t row0, int lane, uint32_t tb,
                                         EpiStage& st) {
+  if (row0 >= M) return;  // none of this warp's rows is masked (warp-uniform)
   const int64_t r = row0 + lane;
   const bool valid = r < M;
   const int32_t y = valid ? p.w.tgt[r] : -1;
@@ -375,12 +391,15 @@ __device__ __forceinline__ void epi_fwd(const GemmParams& p, const CUtensorMap* 
 }
 
 // GEMM_DZ: dz_{r,v} = w_r (1[v = y_r] - e^{z_{r,v} - lse_r}) as bf16, zero for
-// rows >= M and vocabulary columns >= V; 64-column sub-tiles leave through TMA
+// rows in [M, roundup(M, 64)) and vocabulary columns >= V; 64-column sub-tiles leave through TMA
 // stores into dZ [dz_rows, dz_cols], from row `roff` on; vocabulary entry v
 // lands in column v - v_begin + dz_col0.
 __device__ __forceinline__ void epi_dz(const GemmParams& p, const CUtensorMap* map_c, int32_t M,
                                        const Unit& t, int64_t row0, int64_t roff, int lane,
                                        uint32_t tb, EpiStage& st) {
+  // past the dW GEMM's K padding nothing reads dZ: its rows there only reach
+  // accumulator rows of the dX GEMM that no epilogue reads (warp-uniform)
+  if (row0 >= round_up(M, kBK)) return;
   const int64_t r = row0 + lane;
   const bool valid = r < M;
   float w = 0.f, lse_l2 = 0.f;
@@ -448,7 +467,7 @@ __device__ __forceinline__ void epi_dz(const GemmParams& p, const CUtensorMap* m
 // partial buffer, 32-column sub-tiles through TMA stores in the first
 // vocabulary chunk and TMA reduce-adds in the later ones (every element has one
 // writer per launch and the chunks run in order, so the sum is deterministic;
-// rows >= M hold zeros). Without split-K every dX element has exactly this one
+// rows >= M are not read). Without split-K every dX element has exactly this one
 // contribution in the launch, so the lane adds its row's sub-tile straight
 // into dX[b, i] (the row the compaction recorded) with 16-byte atomic adds,
 // which need no round trip: each element still receives one addition, and the
@@ -488,7 +507,7 @@ __device__ __forceinline__ void epi_dx(const GemmParams& p, const CUtensorMap* m
                                        int lane, uint32_t tb, EpiStage& st) {
   const int32_t h0 = nb * kBN;
   const int32_t nsub = min(kBN / 32, ((int32_t)p.g.H - h0 + 31) / 32);  // inside H
-  if (nsub <= 0) return;  // a column block past H (warp-uniform)
+  if (nsub <= 0 || row0 >= M) return;  // a column block past H, no masked row (warp-uniform)
   const int32_t prow0 = (int32_t)(t.split * wk.tiles_m * kPairM + row0);
   const int64_t r = row0 + lane;
   float4* drow = nullptr;
@@ -615,8 +634,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();  // 0: even CTA (issues the MMAs), 1: its peer
   const uint32_t peer = rank ^ 1u;
-  const int64_t pair = blockIdx.x >> 1;
-  const int64_t num_pairs = gridDim.x >> 1;
+  const int32_t pair = (int32_t)(blockIdx.x >> 1);
+  const int32_t num_pairs = (int32_t)(gridDim.x >> 1);
   int32_t* err = p.w.err;
 
   // the prologue touches no global memory: it runs while the kernel before this
@@ -682,18 +701,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       uint32_t phase = 0;
       bool ok = true;
       bool issued = false;
-      for (int64_t u = pair; u < wk.units && ok; u += num_pairs) {
+      for (int32_t u = pair; u < wk.units && ok; u += num_pairs) {
         const Unit t = unit_of<KIND>(wk, u);
         // the even CTA arms the transaction bytes of both CTAs' copies on its
         // full barrier; the odd CTA's copies only complete_tx on it (a
         // per-stage remote arrive from the odd CTA halved the throughput)
         const uint32_t bytes =
-            rank == 0 ? stage_bytes<KIND>(p, t, 0) + stage_bytes<KIND>(p, t, 1) : 0u;
+            rank == 0 ? stage_bytes<KIND>(p, wk, t, 0) + stage_bytes<KIND>(p, wk, t, 1) : 0u;
         for (int32_t kb = t.kb0; kb < t.kb0 + t.kb_n; ++kb) {
           if (!mbar_wait(smem_addr(&empty[stage]), phase ^ 1u, abort_flag)) { ok = false; break; }
           const uint32_t cbar = map_to_cta(smem_addr(&full[stage]), 0);
           if (rank == 0) mbar_arrive_expect_tx(smem_addr(&full[stage]), bytes);
-          load_stage<KIND>(p, &map_a, &map_b, smem_addr(s_a + stage * kTileABytes),
+          load_stage<KIND>(p, wk, &map_a, &map_b, smem_addr(s_a + stage * kTileABytes),
                            smem_addr(s_b + stage * kBBytes), cbar, t, kb, rank, roff);
           issued = true;
           if (++stage == kSt) { stage = 0; phase ^= 1u; }
@@ -720,7 +739,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       uint32_t phase = 0;
       bool ok = true, issued = false;
       int it = 0;
-      for (int64_t u = pair; u < wk.units && ok; u += num_pairs, ++it) {
+      for (int32_t u = pair; u < wk.units && ok; u += num_pairs, ++it) {
         const Unit t = unit_of<KIND>(wk, u);
         const int acc = it % kBufs;
         const uint32_t acc_phase = (uint32_t)(it / kBufs) & 1u;
@@ -778,7 +797,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       prefetch_dw(p, t0, rank, quarter, lane, 0);
       prefetch_dw(p, t0, rank, quarter, lane, 1);
     }
-    for (int64_t u = pair; u < wk.units; u += num_pairs, ++it) {
+    for (int32_t u = pair; u < wk.units; u += num_pairs, ++it) {
       const Unit t = unit_of<KIND>(wk, u);
       const int acc = it % kBufs;
       const uint32_t acc_phase = (uint32_t)(it / kBufs) & 1u;

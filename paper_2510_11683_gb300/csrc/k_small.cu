@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(256) k_lse_combine(Geometry g, int32_t j, bool
 // the logits the forward kept:
 //   dz_{r,v} = w_r (1[v = y_r] - e^{z_{r,v} - lse_r}),  w_r = coef_b / t_b
 // (gradient of Eq. 4 weighted by dL/dl), bf16, zero for rows in
-// [M, round_up(M, 256)) and columns at or past V: the arithmetic of the
+// [M, round_up(M, 64)) and columns at or past V: the arithmetic of the
 // GEMM_DZ epilogue on the same fp32 logits, so both give identical bits.
 // Entry v lands in dZ column v - v0 (a chunk-local buffer) or v (a
 // whole-vocabulary one). HBM-bound: each row streams 4 bytes in and 2 bytes out
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kDzThreads, 4)
   const int64_t zvec = g.v_pad / 8;
   const int64_t dvec = w.dz_cols / 8;
   const int64_t per_row = ceil_div(nvec, kDzItemVecs);
-  const int64_t items = round_up(M, kPairM) * per_row;
+  const int64_t items = round_up(M, kBK) * per_row;   // rows the dW GEMM's K blocks read
   const float4* zc = reinterpret_cast<const float4*>(w.zc) + v_begin / 4;
   // this sample's dZ rows start at the pairing offset (0 without pairing)
   uint4* dz = reinterpret_cast<uint4*>(w.dz) +
