@@ -408,32 +408,84 @@ __global__ void k_vrpo_coeffs(int32_t B, int32_t n_t, float loss_scale, const fl
 // ---------------------------------------------------------------------------
 // dX[b, i, :] += sum_s partial_s[r, :] over the split-K partials of the dX GEMM
 // (fixed split order; rows are unique within a sample, so no atomics). With a
-// single split the GEMM's epilogue has already added its tile into dX. Each
-// thread keeps kDxrVec 16-byte loads of a split (and of the dX row) in flight
-// at once.
+// single split the GEMM's epilogue has already added its tile into dX. Above
+// H = 2048 a block takes one row, four 16-byte loads of a split per thread in
+// flight. Below, a row is too little for a block: the M H / 4 vectors are cut
+// into flat tiles of 1,024, or of 256 with four splits' loads in flight where
+// 1,024 would leave SMs without a block. One block per row there took (-> now)
+// 24 -> 6.0 us at 4,000 rows of 128, 16 -> 4.9 at 3,310 of 256, 5.5 -> 3.4 at 420
+// of 512, 16.5 -> 10.3 at 2,000 of 1,024, 8.4 -> 7.1 at 495 of 1,536; above, the
+// flat tiles' row lookups cost 12.9 -> 14.5 us at 1,000 rows of 4,096.
 // ---------------------------------------------------------------------------
 constexpr int kDxrThreads = 256;
 constexpr int kDxrVec = 4;
+constexpr int64_t kDxrRowVecs = 512;        // 16-byte vectors of a row above which a block takes it
+constexpr int64_t kDxrFlatTiles = 160;      // fewest tiles of 1,024 vectors
+constexpr int64_t kDxrFlatBlocks = 2432;    // 16 per SM of 152
 
-__global__ void __launch_bounds__(kDxrThreads) k_dx_reduce(Geometry g, int32_t j, WsPtrs w,
-                                                           float* dX) {
-  pdl_begin();
-  const int32_t M = rows_of_sample(w.err, j, KID_DX_REDUCE);
-  const int64_t r = blockIdx.x;
-  if (r >= M) return;
-  const int64_t mb = ceil_div(M, kPairM);
-  const int S = w.err[ERR_DX_SPLITS];  // written by the dX GEMM of this sample
-  if (S == 1) return;
-  if (S < 1 || S > kMaxSplits || S * mb > dxp_row_block_cap(g)) {  // not a count it can write
-    if (r == 0 && threadIdx.x == 0) set_device_error(w.err, kStatusInvalidArg, KID_DX_REDUCE * 16 + 2);
-    return;
+template <int VEC>
+__device__ __forceinline__ void dx_reduce_tile(const Geometry& g, const WsPtrs& w, float4* dX,
+                                               int64_t tile, int64_t M, int S,
+                                               int64_t split_stride) {
+  const uint32_t nvec = (uint32_t)(g.H / 4);
+  const int64_t v0 = tile * (kDxrThreads * VEC);
+  const int64_t r0 = v0 / nvec;
+  const uint32_t c0 = (uint32_t)(v0 - r0 * nvec);
+  const float4* src = reinterpret_cast<const float4*>(w.dxp) + v0;
+  float4 acc[VEC], o[VEC];
+  float4* dst[VEC];
+#pragma unroll
+  for (int k = 0; k < VEC; ++k) {
+    const uint32_t h = threadIdx.x + (uint32_t)k * kDxrThreads;
+    const uint32_t x = c0 + h;
+    const int64_t r = r0 + x / nvec;
+    dst[k] = nullptr;
+    if (r < M) {
+      const int32_t idx = w.rows[r];
+      if (BGPO_IN_BOUNDS(w.err, idx >= 0 && idx < g.m_cap, KID_DX_REDUCE * 16 + 9))
+        dst[k] = dX + (int64_t)idx * nvec + x % nvec;
+    }
   }
-  const int64_t split_stride = mb * kPairM * g.H / 4;
+  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int k = 0; k < VEC; ++k)
+    acc[k] = dst[k] ? src[threadIdx.x + k * kDxrThreads] : z;
+#pragma unroll
+  for (int k = 0; k < VEC; ++k) o[k] = dst[k] ? *dst[k] : z;
+  constexpr int kBatch = kDxrVec / VEC;   // splits whose loads are in flight together
+  for (int s0 = 1; s0 < S; s0 += kBatch) {
+    float4 v[kBatch][VEC];
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q)
+#pragma unroll
+      for (int k = 0; k < VEC; ++k)
+        v[q][k] = (dst[k] && s0 + q < S)
+                      ? src[(s0 + q) * split_stride + threadIdx.x + k * kDxrThreads] : z;
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q)
+      if (s0 + q < S) {
+#pragma unroll
+        for (int k = 0; k < VEC; ++k) {
+          acc[k].x += v[q][k].x; acc[k].y += v[q][k].y;
+          acc[k].z += v[q][k].z; acc[k].w += v[q][k].w;
+        }
+      }
+  }
+#pragma unroll
+  for (int k = 0; k < VEC; ++k)
+    if (dst[k]) {
+      o[k].x += acc[k].x; o[k].y += acc[k].y; o[k].z += acc[k].z; o[k].w += acc[k].w;
+      *dst[k] = o[k];
+    }
+}
+
+__device__ __forceinline__ void dx_reduce_row(const Geometry& g, const WsPtrs& w, float4* dX,
+                                              int64_t r, int S, int64_t split_stride) {
   const int32_t idx = w.rows[r];
   if (!BGPO_IN_BOUNDS(w.err, idx >= 0 && idx < g.m_cap, KID_DX_REDUCE * 16 + 9)) return;
-  const float4* src = reinterpret_cast<const float4*>(w.dxp) + r * (g.H / 4);
-  float4* dst = reinterpret_cast<float4*>(dX) + (int64_t)idx * (g.H / 4);
   const int64_t nvec = g.H / 4;
+  const float4* src = reinterpret_cast<const float4*>(w.dxp) + r * nvec;
+  float4* dst = dX + (int64_t)idx * nvec;
   for (int64_t h0 = threadIdx.x; h0 < nvec; h0 += (int64_t)kDxrThreads * kDxrVec) {
     float4 acc[kDxrVec], o[kDxrVec];
 #pragma unroll
@@ -463,6 +515,35 @@ __global__ void __launch_bounds__(kDxrThreads) k_dx_reduce(Geometry g, int32_t j
         dst[h] = o[k];
       }
     }
+  }
+}
+
+__global__ void __launch_bounds__(kDxrThreads) k_dx_reduce(Geometry g, int32_t j, WsPtrs w,
+                                                           float* dX) {
+  pdl_begin();
+  const int64_t M = rows_of_sample(w.err, j, KID_DX_REDUCE);
+  const int64_t mb = ceil_div(M, kPairM);
+  const int S = w.err[ERR_DX_SPLITS];  // written by the dX GEMM of this sample
+  if (S == 1 || M <= 0) return;
+  if (S < 1 || S > kMaxSplits || S * mb > dxp_row_block_cap(g)) {  // not a count it can write
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+      set_device_error(w.err, kStatusInvalidArg, KID_DX_REDUCE * 16 + 2);
+    return;
+  }
+  const int64_t split_stride = mb * kPairM * g.H / 4;
+  const int64_t nvec = g.H / 4;
+  float4* out = reinterpret_cast<float4*>(dX);
+  if (nvec > kDxrRowVecs) {
+    const int64_t r = blockIdx.x;
+    if (r < M) dx_reduce_row(g, w, out, r, S, split_stride);
+  } else if (M * nvec >= kDxrFlatTiles * kDxrVec * kDxrThreads) {
+    const int64_t tiles = ceil_div(M * nvec, kDxrVec * kDxrThreads);
+    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x)
+      dx_reduce_tile<kDxrVec>(g, w, out, t, M, S, split_stride);
+  } else {
+    const int64_t tiles = ceil_div(M * nvec, kDxrThreads);
+    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x)
+      dx_reduce_tile<1>(g, w, out, t, M, S, split_stride);
   }
 }
 
@@ -655,7 +736,12 @@ cudaError_t launch_vrpo_coeffs(int32_t B, int32_t n_t, float loss_scale, const f
 
 cudaError_t launch_dx_reduce(const Geometry& g, int32_t j, const WsPtrs& w, float* dX,
                              cudaStream_t s) {
-  return launch_dependent(k_dx_reduce, (unsigned)g.m_cap, kDxrThreads, 0, s, g, j, w, dX);
+  int64_t grid = g.m_cap;
+  if (g.H / 4 <= kDxrRowVecs) {
+    grid = ceil_div(g.m_cap * (g.H / 4), kDxrThreads);
+    if (grid > kDxrFlatBlocks) grid = kDxrFlatBlocks;
+  }
+  return launch_dependent(k_dx_reduce, (unsigned)grid, kDxrThreads, 0, s, g, j, w, dX);
 }
 
 cudaError_t launch_xm_transpose(const Geometry& g, int32_t j, bool defer, const WsPtrs& w,
