@@ -371,7 +371,7 @@ bgpo_status bgpo_elbo_bwd_accumulate(const bgpo_problem* prob, int32_t j, const 
   {
     // Xm^T for the dW GEMMs; also records the dW pairing state of this sample
     TraceScope ts(prob->trace, KID_XM_TRANSPOSE, s);
-    if (launch_xm_transpose(g, j, defer, w, s) != cudaSuccess) return BGPO_ERR_CUDA;
+    if (launch_xm_transpose(g, j, defer, ga.num_pairs, w, s) != cudaSuccess) return BGPO_ERR_CUDA;
   }
   // One vocabulary chunk at a time (Linearity, Sec. 3, within a sample: the
   // gradient is a sum over vocabulary entries too): dZ of the chunk, its dX

@@ -88,9 +88,10 @@ cudaError_t launch_dx_reduce(const Geometry& g, int32_t j, const WsPtrs& w, floa
                              cudaStream_t s);
 // Xm^T from Xm for the current sample's rows (the dW GEMM reads it K-major),
 // from column ERR_ROW_OFF on. `defer`: this sample's dW GEMM waits for the
-// next sample's; the kernel records the sample as pending.
-cudaError_t launch_xm_transpose(const Geometry& g, int32_t j, bool defer, const WsPtrs& w,
-                                cudaStream_t s);
+// next sample's; the kernel records the sample as pending. It also leaves the
+// dX GEMM's plan for `num_pairs` CTA pairs.
+cudaError_t launch_xm_transpose(const Geometry& g, int32_t j, bool defer, int num_pairs,
+                                const WsPtrs& w, cudaStream_t s);
 cudaError_t launch_group_advantage(int32_t B, int32_t G, const float* rewards, float* A_out,
                                    cudaStream_t s);
 cudaError_t launch_vrpo_coeffs(int32_t B, int32_t n_t, float loss_scale, const float* ell,

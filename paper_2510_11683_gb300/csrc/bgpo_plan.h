@@ -24,18 +24,16 @@ constexpr int kBNHalf = 128;     // B columns staged by each CTA of the pair
 constexpr int kBK = 64;          // K per pipeline stage: one 128-byte swizzle row of bf16
 constexpr int kUmmaK = 16;       // K of one tcgen05.mma kind::f16 instruction
 constexpr int kStages = 6;       // TMA -> MMA pipeline depth
-// The dX GEMM's tiles are kDxWide accumulators wide (256 x 512 for 2): each
-// K block of A then feeds kDxWide MMAs, so the operand stream per flop into
+// The dX GEMM's tiles are one or two accumulators wide (dx_plan). Two (256 x
+// 512): each K block of A feeds two MMAs, so the operand stream per flop into
 // shared memory is 3/4 of a 256 x 256 tile's, and a wave of tiles covers all
-// of H with half as many W column blocks re-read per row block. Both of the
+// of H with half as many W column blocks re-read per row block; both of the
 // pair's 256-column accumulators hold one tile (the epilogue does not overlap
-// the next tile's main loop), with kDxStages stages of 48 KB per CTA.
-#ifndef BGPO_DX_WIDE
-#define BGPO_DX_WIDE 2
-#endif
-constexpr int kDxWide = BGPO_DX_WIDE;
-static_assert(kDxWide == 1 || kDxWide == 2, "dX tile width: one or two accumulators");
-constexpr int kDxStages = kDxWide == 2 ? 4 : kStages;
+// the next tile's main loop), with kDxStages stages of 48 KB per CTA. One: the
+// other GEMMs' kStages stages of 32 KB in the same shared memory.
+constexpr int kDxWide = 2;
+constexpr int kDxStages = 4;
+static_assert(kDxStages * (1 + kDxWide) == kStages * 2, "both stage rings fill the same bytes");
 constexpr int kMaxSplits = 16;   // split-K limit of the dX GEMM
 // Widest vocabulary chunk of the backward by default: dZ is formed, used by
 // the dX GEMM and the dW GEMM one chunk of at most this many columns at a
@@ -77,8 +75,9 @@ enum KernelId : int32_t {
 BGPO_HD int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 BGPO_HD int64_t round_up(int64_t a, int64_t b) { return ceil_div(a, b) * b; }
 
-// Column tiles of the dX GEMM for `tiles_h` hidden-size blocks of kBN columns.
-BGPO_HD int64_t dx_tiles_n(int64_t tiles_h) { return ceil_div(tiles_h, kDxWide); }
+// Column tiles of the dX GEMM for `tiles_h` hidden-size blocks of kBN columns,
+// `wide` of them per tile.
+BGPO_HD int64_t dx_tiles_n(int64_t tiles_h, int wide = kDxWide) { return ceil_div(tiles_h, wide); }
 
 // Row groups of the forward and dZ GEMMs. Consecutive tiles share a vocabulary
 // tile of W, so every wave of tiles reads all of Xm's row blocks; once Xm
@@ -249,6 +248,73 @@ BGPO_HD int64_t dxp_row_block_cap(const Geometry& g) {
   return cap > kMaxSplits ? cap : kMaxSplits;
 }
 
+// Tile width and split count of the dX GEMM of a sample with M masked rows (the
+// same for every chunk of the sample): 256 x 512 tiles split by dx_splits, unless
+// another pair of the two is estimated to take at least 5% less (dx_cost). That is
+// so where a split's K loop is short against its epilogue and its partials, and
+// where H leaves a second accumulator empty. GEMM and reduction, 512-wide tiles
+// -> now, in us: M 291, H 152, V 137580: 153 -> 113; M 4398, H 104, V 84350: 247 ->
+// 183; M 300, H 1024, V 8192: 22.1 -> 17.4; M 5331, H 2712, V 975 (split twice ->
+// unsplit): 116 -> 62; M 110, H 808, V 14743 in chunks of 1,024: 185 -> 132. Over
+// 36 shapes drawn from H 64 .. 4096, V 512 .. 152,064, 1 .. 16,384 response rows
+// the geometric mean is 1.22 times faster and none is slower by more than 1%. Over
+// vocabulary chunks, where every split's partial is read and written again for
+// each chunk, fewer splits win (against the time of the same sample's dZ GEMM,
+// which the power cap slows alike): H 3584, V 152064, 5 chunks: 1.29 times faster
+// at 1,259 rows (13 -> 2 splits), 1.11 at 4,893, 1.02 at 10,165, 0.99 at 12,489;
+// H 4096, V 126464, 4 chunks: 1.04 at 951 rows, 1.06 at 2,027, 1.03 at 4,286.
+struct DxPlan {
+  int32_t wide, splits;
+};
+
+// Estimated cycles of the GEMM over all chunks and of the split reduction. The
+// constants are fits to 15 shapes times 10 forced plans, measured on a GB300 at
+// about 2 GHz: a K block takes 700 cycles at one accumulator and 1,030 at two, a
+// launch 16,000 and 19,200 beside its K loops; at two, each further wave shows its
+// epilogue; unsplit tiles, which add into dX themselves, take 12,000 and 17,400
+// longer; partials stream at 3,100 bytes per cycle.
+BGPO_HD float dx_cost(const Geometry& g, int64_t M, int num_pairs, int wide, int s) {
+  const uint32_t units =
+      (uint32_t)(ceil_div(M, kPairM) * dx_tiles_n(g.tiles_h, wide)) * (uint32_t)s;
+  const float waves = (float)((units + (uint32_t)num_pairs - 1) / (uint32_t)num_pairs);
+  const float kb = (float)(((uint32_t)g.kb_vc_min + (uint32_t)s - 1) / (uint32_t)s);
+  float gemm = waves * kb * (wide == 1 ? 700.f : 1030.f);
+  gemm += wide == 1 ? 16000.f : 9200.f + 10000.f * waves;
+  if (s == 1) gemm += wide == 1 ? 12000.f : 17400.f * waves;
+  // passes over M x H floats: each partial once and dX twice in the reduction, and
+  // each partial twice for every chunk that adds to it
+  const float passes = (float)(s + 2 + 2 * s * (int)(g.n_vc - 1));
+  const float reduce = s == 1 ? 2600.f : 4000.f + passes * (float)M * (float)g.H * (4.f / 3100.f);
+  return gemm * (float)g.n_vc + reduce;
+}
+
+// Candidate i of the 32: a tile width and a split count the split buffer has room for.
+BGPO_HD DxPlan dx_candidate(int i) { return DxPlan{1 + (i & 1), 1 + (i >> 1)}; }
+BGPO_HD bool dx_fits(const Geometry& g, int64_t M, const DxPlan& c) {
+  return c.splits <= g.kb_vc_min && c.splits * ceil_div(M, kPairM) <= dxp_row_block_cap(g);
+}
+
+// The plan, given the candidate of least cost (M > 0).
+BGPO_HD DxPlan dx_plan_of(const Geometry& g, int64_t M, int num_pairs, const DxPlan& best,
+                          float cost) {
+  const DxPlan usual = {kDxWide, dx_splits(ceil_div(M, kPairM), dx_tiles_n(g.tiles_h), num_pairs,
+                                           g.kb_vc_min, dxp_row_block_cap(g))};
+  return cost <= 0.95f * dx_cost(g, M, num_pairs, usual.wide, usual.splits) ? best : usual;
+}
+
+BGPO_HD DxPlan dx_plan(const Geometry& g, int64_t M, int num_pairs) {
+  if (M <= 0) return DxPlan{kDxWide, 1};
+  DxPlan best = dx_candidate(0);   // one split always fits
+  float cost = dx_cost(g, M, num_pairs, best.wide, best.splits);
+  for (int i = 1; i < 2 * kMaxSplits; ++i) {
+    const DxPlan c = dx_candidate(i);
+    if (!dx_fits(g, M, c)) continue;
+    const float t = dx_cost(g, M, num_pairs, c.wide, c.splits);
+    if (t < cost) { cost = t; best = c; }
+  }
+  return dx_plan_of(g, M, num_pairs, best, cost);
+}
+
 // `keep_logits` appends the fp32 logit region. `pair_dw` doubles the rows of
 // dZ and the columns of Xm^T: the rows of an even sample wait there for the
 // dW GEMM of the next sample, whose rows follow them; its dZ rows then span
@@ -288,7 +354,8 @@ BGPO_HD WsLayout make_ws_layout(const Geometry& g, bool keep_logits, bool pair_d
 //   ERR_LOGITS    1 while the logit region holds the current sample's logits
 //                 (set by the forward that wrote them, cleared by the masking of
 //                 a new sample and by a forward that keeps none)
-//   ERR_DX_SPLITS the split-K count the last dX GEMM used
+//   ERR_DX_SPLITS, ERR_DX_WIDE  the plan of the current sample's dX GEMM (DxPlan), set by
+//                 the backward's first kernel
 //   ERR_PEND      pend_tag(j) while sample j's dZ and Xm^T rows wait for the dW
 //                 GEMM of sample j + 1, else -1
 //   ERR_PEND_OFF  the row at which sample j + 1's dZ and Xm^T rows start: M_j
@@ -302,7 +369,8 @@ BGPO_HD WsLayout make_ws_layout(const Geometry& g, bool keep_logits, bool pair_d
 //                 an earlier backward of this sample has added the partner)
 enum ErrField : int {
   ERR_STATUS = 0, ERR_WHERE = 1, ERR_SAMPLE = 2, ERR_M = 3, ERR_LOGITS = 4, ERR_DX_SPLITS = 5,
-  ERR_PEND = 6, ERR_PEND_OFF = 7, ERR_ROW_OFF = 8, ERR_PAIRED = 9, ERR_DW_K0 = 10
+  ERR_PEND = 6, ERR_PEND_OFF = 7, ERR_ROW_OFF = 8, ERR_PAIRED = 9, ERR_DW_K0 = 10,
+  ERR_DX_WIDE = 11
 };
 
 // Tag of a pending sample (n_t < 2^16): neither -1 nor a small integer that

@@ -4,10 +4,10 @@
 // CTA pair computes 256 x 256 fp32 tiles with tcgen05.mma.cta_group::2: CTA r
 // of the pair stages rows [128 r, 128 r + 128) of the A tile and columns
 // [128 r, 128 r + 128) of the B tile, and holds accumulator rows
-// [128 r, 128 r + 128) in its TMEM. The dX GEMM's tiles are kDxWide such
+// [128 r, 128 r + 128) in its TMEM. The dX GEMM's tiles are one or two such
 // tiles side by side, sharing their A tile. Roles in each CTA (192 threads):
 //   warp 0      TMA producer: 128-byte-swizzled bf16 boxes into a 6-stage ring
-//               of 32 KB (dX: 4 stages of 48 KB); every copy of both CTAs completes on the even CTA's
+//               of 32 KB (dX at two: 4 stages of 48 KB); every copy of both CTAs completes on the even CTA's
 //               "full" barrier, which the even CTA alone arms with both CTAs'
 //               transaction bytes (a negative transaction count in between is
 //               allowed)
@@ -28,7 +28,7 @@
 //             vocabulary chunk of the backward; epilogue: dz = w_r (onehot -
 //             e^{z - lse}) stored as bf16 (gradient of Eq. 4 weighted by
 //             Eq. 13's dL/dl).
-//   GEMM_DX   dXm += dZ_c W_c (K = the chunk's vocabulary; 256 x 512 tiles): split-K partials in
+//   GEMM_DX   dXm += dZ_c W_c (K = the chunk's vocabulary; 256 x 256 or 256 x 512 tiles): split-K partials in
 //             fp32, stored by the first chunk and added by the later ones, or,
 //             when the launch needs no split, added straight into the dX rows.
 //   GEMM_DW   dW[chunk rows] += dZ_c^T Xm (K = masked rows; Xm read as its
@@ -76,6 +76,7 @@ struct Work {
   int32_t kb_first;  // first K block (dW: a partner already added is skipped)
   int32_t groups;    // forward and dZ: row groups (xm_row_groups)
   int32_t splits;
+  int32_t wide;      // accumulators per tile (dX: one or two)
   int32_t rows;      // A rows that hold data: CTAs and warps wholly past them skip theirs
 };
 
@@ -91,6 +92,7 @@ __device__ __forceinline__ Work make_work(const GemmParams& p, int32_t M, int64_
                                           int64_t k0) {
   Work w;
   w.splits = 1;
+  w.wide = 1;
   w.kb_first = 0;
   w.groups = 1;
   w.rows = M;
@@ -103,13 +105,14 @@ __device__ __forceinline__ Work make_work(const GemmParams& p, int32_t M, int64_
     w.groups = (int32_t)xm_row_groups(w.tiles_m, p.g.H);
   } else if (KIND == GEMM_DX) {
     w.tiles_m = (int32_t)ceil_div(M, kPairM);
-    w.tiles_n = (int32_t)dx_tiles_n(p.g.tiles_h);
     w.kb_total = (int32_t)ceil_div(p.v_end - p.v_begin, kBK);
-    // one split count for every chunk of the sample (the partials of split s
-    // accumulate over the chunks), bounded by the narrowest chunk's K blocks
-    w.splits = w.tiles_m > 0 ? dx_splits(w.tiles_m, w.tiles_n, p.num_pairs, p.g.kb_vc_min,
-                                         dxp_row_block_cap(p.g))
-                             : 1;
+    // one plan for every chunk of the sample (the partials of split s
+    // accumulate over the chunks), left by the kernel that transposed Xm
+    const DxPlan plan = {p.w.err[ERR_DX_WIDE], p.w.err[ERR_DX_SPLITS]};
+    const bool fits = plan.splits >= 1 && plan.splits <= kMaxSplits && dx_fits(p.g, M, plan);
+    w.wide = plan.wide == 1 ? 1 : kDxWide;
+    w.splits = fits ? plan.splits : 1;
+    w.tiles_n = (int32_t)dx_tiles_n(p.g.tiles_h, w.wide);
     w.units = w.tiles_m * w.tiles_n * w.splits;
   } else {  // GEMM_DW
     w.tiles_m = (int32_t)ceil_div(p.v_end - p.v_begin, kPairM);
@@ -156,23 +159,13 @@ __device__ __forceinline__ Unit unit_of(const Work& w, int32_t u) {
   return t;
 }
 
-// Shared-memory plan of one kind: 6 pipeline stages and the epilogue's
-// staging buffers (the forward GEMM stages its fp32 logits there when it keeps
-// them).
-template <int KIND>
-struct Shape {
-  static constexpr int nacc = KIND == GEMM_DX ? kDxWide : 1;  // accumulators per tile
-  static constexpr int bufs = 2 / nacc;                        // tiles in TMEM at once
-  static constexpr int stages = KIND == GEMM_DX ? kDxStages : kStages;
-  static constexpr uint32_t b_bytes = nacc * kTileBBytes;      // B bytes per CTA and stage
-};
-
+// Shared-memory plan of one kind: 6 pipeline stages (dX with two accumulators
+// per tile: 4 larger ones in the same bytes) and the epilogue's staging buffers
+// (the forward GEMM stages its fp32 logits there when it keeps them).
 template <int KIND>
 struct SmemPlan {
-  static constexpr int stages = Shape<KIND>::stages;
   static constexpr uint32_t epi_bytes = kEpiBytes;
-  static constexpr uint32_t bytes =
-      stages * (kTileABytes + Shape<KIND>::b_bytes) + epi_bytes + 1024 + 1024;
+  static constexpr uint32_t bytes = kStages * kStageBytes + epi_bytes + 1024 + 1024;
   static_assert(bytes <= 232448, "shared memory per CTA");
 };
 
@@ -230,7 +223,7 @@ __device__ __forceinline__ LoadPlan load_plan(const GemmParams& p, const Work& w
   LoadPlan q;
   const int32_t a0 = t.m_blk * kPairM + (int32_t)rank * kBM;
   const int64_t b0 =
-      b_base<KIND>(p) + (int64_t)t.n_blk * Shape<KIND>::nacc * kBN + (int64_t)rank * kBNHalf;
+      b_base<KIND>(p) + (int64_t)t.n_blk * w.wide * kBN + (int64_t)rank * kBNHalf;
   if (!Majors<KIND>::a_mn) {
     q.a_x = KIND == GEMM_DX ? (int32_t)p.dz_col0 : 0;
     q.a_y = a0 + (KIND == GEMM_DX ? (int32_t)roff : 0);
@@ -252,7 +245,7 @@ __device__ __forceinline__ LoadPlan load_plan(const GemmParams& p, const Work& w
     q.b_x = (int32_t)b0;
     q.b_y = (int32_t)p.v_begin;
     q.b_boxes = 0;
-    for (int i = 0; i < 2 * Shape<KIND>::nacc; ++i)
+    for (int i = 0; i < 2 * w.wide; ++i)
       if (b0 + (i >> 1) * kBN + (i & 1) * 64 < p.g.H) q.b_boxes = i + 1;
   }
   return q;
@@ -508,30 +501,42 @@ __device__ __forceinline__ void epi_dz(const GemmParams& p, const CUtensorMap* m
 // vocabulary chunk and TMA reduce-adds in the later ones (every element has one
 // writer per launch and the chunks run in order, so the sum is deterministic;
 // rows >= M are not read). Without split-K every dX element has exactly this one
-// contribution in the launch, so the lane adds its row's sub-tile straight
-// into dX[b, i] (the row the compaction recorded) with 16-byte atomic adds,
-// which need no round trip: each element still receives one addition, and the
-// split reduction after the last chunk has nothing to do.
+// contribution in the launch, so the warp adds its sub-tile straight into the
+// rows dX[b, i] (which the compaction recorded) with 16-byte atomic adds, which
+// need no round trip: each element still receives one addition, and the split
+// reduction after the last chunk has nothing to do. The sub-tile is turned in the
+// staging buffer first, so that one instruction adds four rows' whole 128-byte
+// lines instead of 16 bytes of 32 rows: 1,000 rows of 4,096, K = 2,000: 45.6 -> 25.8
+// us with 256 x 256 tiles, 1,500 of 3,000, K = 12,000: 117 -> 87.
 __device__ __forceinline__ void dx_sub(const GemmParams& p, const CUtensorMap* map_c,
-                                       const Work& wk, float4* drow, int32_t h0, int32_t prow0,
+                                       const Work& wk, const RowInfo& q, int32_t h0, int32_t prow0,
                                        int c, const uint32_t (&raw)[32], int lane, EpiStage& st) {
-  if (wk.splits == 1) {  // launch-uniform
-    if (drow) {
-      // 16-byte pieces of this sub-tile inside the row (H is a multiple of 8)
-      const int nq = min(8, ((int32_t)p.g.H - (h0 + c * 32)) / 4);
+  uint4 chunk[8];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        if (q >= nq) break;
-        atomicAdd(drow + c * 8 + q, make_float4(bits_f(raw[4 * q]), bits_f(raw[4 * q + 1]),
-                                                bits_f(raw[4 * q + 2]), bits_f(raw[4 * q + 3])));
+  for (int e = 0; e < 8; ++e)
+    chunk[e] = make_uint4(raw[4 * e], raw[4 * e + 1], raw[4 * e + 2], raw[4 * e + 3]);
+  if (wk.splits == 1) {  // launch-uniform
+    const uint32_t buf = st.base + (uint32_t)(c & 1) * kEpiBufBytes;
+    stage_row(buf, lane, chunk);
+    __syncwarp();
+    // 16-byte piece of this lane inside each row (H is a multiple of 8)
+    const int32_t col = h0 + c * 32 + (lane & 7) * 4;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int row = 4 * k + (lane >> 3);
+      const int32_t pos = __shfl_sync(0xffffffffu, q.pos, row);
+      if (pos >= 0 && col < (int32_t)p.g.H) {
+        float4 v;
+        const uint32_t a = buf + (uint32_t)row * 128u + (uint32_t)(((lane & 7) ^ (row & 7)) * 16);
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                     : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                     : "r"(a)
+                     : "memory");
+        atomicAdd(reinterpret_cast<float4*>(p.dX + (int64_t)pos * p.g.H + col), v);
       }
     }
     return;
   }
-  uint4 chunk[8];
-#pragma unroll
-  for (int q = 0; q < 8; ++q)
-    chunk[q] = make_uint4(raw[4 * q], raw[4 * q + 1], raw[4 * q + 2], raw[4 * q + 3]);
   const uint32_t sbuf = st.acquire(lane);
   stage_row(sbuf, lane, chunk);
   if (p.chunk == 0)
@@ -549,19 +554,17 @@ __device__ __forceinline__ void epi_dx(const GemmParams& p, const CUtensorMap* m
   const int32_t nsub = min(kBN / 32, ((int32_t)p.g.H - h0 + 31) / 32);  // inside H
   if (nsub <= 0 || row0 >= M) return;  // a column block past H, no masked row (warp-uniform)
   const int32_t prow0 = (int32_t)(t.split * wk.tiles_m * kPairM + row0);
-  float4* drow = nullptr;
-  if (q.pos >= 0) drow = reinterpret_cast<float4*>(p.dX + (int64_t)q.pos * p.g.H + h0);
   uint32_t ra[32], rb[32];
   tmem_ld_32x32b_x32(tb, ra);
   tmem_ld_wait_regs(ra);
 #pragma unroll 1
   for (int c = 0; c < nsub; c += 2) {
     if (c + 1 < nsub) tmem_ld_32x32b_x32(tb + (uint32_t)(c + 1) * 32, rb);
-    dx_sub(p, map_c, wk, drow, h0, prow0, c, ra, lane, st);
+    dx_sub(p, map_c, wk, q, h0, prow0, c, ra, lane, st);
     if (c + 1 < nsub) {
       tmem_ld_wait_regs(rb);
       if (c + 2 < nsub) tmem_ld_32x32b_x32(tb + (uint32_t)(c + 2) * 32, ra);
-      dx_sub(p, map_c, wk, drow, h0, prow0, c + 1, rb, lane, st);
+      dx_sub(p, map_c, wk, q, h0, prow0, c + 1, rb, lane, st);
       if (c + 2 < nsub) tmem_ld_wait_regs(ra);
     }
   }
@@ -647,20 +650,15 @@ template <int KIND>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     k_gemm(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
            const __grid_constant__ CUtensorMap map_c, const GemmParams p) {
-  constexpr int kSt = SmemPlan<KIND>::stages;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
-  constexpr uint32_t kBBytes = Shape<KIND>::b_bytes;
-  constexpr int kNacc = Shape<KIND>::nacc;
-  constexpr int kBufs = Shape<KIND>::bufs;
-  uint8_t* s_a = smem;
-  uint8_t* s_b = smem + kSt * kTileABytes;
-  uint8_t* s_epi = s_b + kSt * kBBytes;   // 4 warps x 2 staging buffers
+  constexpr int kSt = kStages;            // barriers; the dX GEMM may use fewer stages
+  uint8_t* s_epi = smem + kStages * kStageBytes;   // 4 warps x 2 staging buffers
   uint64_t* bars = reinterpret_cast<uint64_t*>(s_epi + SmemPlan<KIND>::epi_bytes);
   uint64_t* full = bars;                      // [kSt] TMA (both CTAs) -> MMA; even CTA's
-  uint64_t* empty = bars + kSt;           // [kSt] MMA -> TMA of each CTA
-  uint64_t* tfull = bars + 2 * kSt;       // [2] MMA -> epilogue of each CTA
+  uint64_t* empty = bars + kSt;               // [kSt] MMA -> TMA of each CTA
+  uint64_t* tfull = bars + 2 * kSt;           // [2] MMA -> epilogue of each CTA
   uint64_t* tempty = bars + 2 * kSt + 2;  // [2] epilogues (both CTAs) -> MMA; even CTA's
   uint64_t* done = bars + 2 * kSt + 4;    // MMA drain on abort
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kSt + 5);
@@ -728,8 +726,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       set_device_error(err, kStatusInvalidArg, kernel_id<KIND>() * 16 + 5);
     err[ERR_PEND] = -1;  // nothing waits any more
   }
-  // the split reduction after the dX GEMM reads the split count from here
-  if (KIND == GEMM_DX && blockIdx.x == 0 && threadIdx.x == 0) err[ERR_DX_SPLITS] = wk.splits;
+  // tiles of two accumulators fill TMEM (one tile at a time) and take 48 KB a stage
+  const int wide = KIND == GEMM_DX ? wk.wide : 1;
+  const int nst = wide == 2 ? kDxStages : kStages;
+  const uint32_t b_bytes = (uint32_t)wide * kTileBBytes;
+  uint8_t* s_a = smem;
+  uint8_t* s_b = smem + nst * kTileABytes;
 
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs) ----------------
@@ -752,10 +754,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         for (int32_t k = t.kb0 * kBK, end = (t.kb0 + t.kb_n) * kBK; k < end; k += kBK) {
           if (!mbar_wait(empty0 + stage * 8, phase ^ 1u, abort_flag)) { ok = false; break; }
           if (rank == 0) mbar_arrive_expect_tx(full0 + stage * 8, bytes);
-          load_stage<KIND>(lp, &map_a, &map_b, sa0 + stage * kTileABytes, sb0 + stage * kBBytes,
+          load_stage<KIND>(lp, &map_a, &map_b, sa0 + stage * kTileABytes, sb0 + stage * b_bytes,
                            cfull0 + stage * 8, k);
           issued = true;
-          if (++stage == kSt) { stage = 0; phase ^= 1u; }
+          if (++stage == nst) { stage = 0; phase ^= 1u; }
         }
       }
       if (!ok) {
@@ -788,8 +790,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       int it = 0;
       for (int32_t u = pair; u < wk.units && ok; u += num_pairs, ++it) {
         const Unit t = unit_of<KIND>(wk, u);
-        const int acc = it % kBufs;
-        const uint32_t acc_phase = (uint32_t)(it / kBufs) & 1u;
+        const int acc = wide == 2 ? 0 : it & 1;
+        const uint32_t acc_phase = (uint32_t)(wide == 2 ? it : it >> 1) & 1u;
         if (!mbar_wait(smem_addr(&tempty[acc]), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * kBN);
@@ -799,18 +801,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           // the address fields of the descriptors count 16-byte units and never
           // carry out of their 14 bits (shared memory is below 2^18 bytes)
           const uint64_t ad = a_desc + (uint64_t)((uint32_t)stage * (kTileABytes >> 4));
-          const uint64_t bd = b_desc + (uint64_t)((uint32_t)stage * (kBBytes >> 4));
+          const uint64_t bd = b_desc + (uint64_t)((uint32_t)stage * (b_bytes >> 4));
+          if (KIND == GEMM_DX && wide == 2) {
 #pragma unroll
-          for (int k = 0; k < kBK / kUmmaK; ++k)
+            for (int k = 0; k < kBK / kUmmaK; ++k) {
+              const uint32_t add = (kb > 0 || k > 0) ? 1u : 0u;
+              umma_bf16_pair(d_tmem, ad + k * kAStep, bd + k * kBStep, idesc, add);
+              umma_bf16_pair(d_tmem + kBN, ad + k * kAStep, bd + (kTileBBytes >> 4) + k * kBStep,
+                             idesc, add);
+            }
+          } else {
 #pragma unroll
-            for (int g = 0; g < kNacc; ++g)
-              umma_bf16_pair(d_tmem + (uint32_t)(g * kBN), ad + k * kAStep,
-                             bd + (uint64_t)g * (kTileBBytes >> 4) + k * kBStep, idesc,
+            for (int k = 0; k < kBK / kUmmaK; ++k)
+              umma_bf16_pair(d_tmem, ad + k * kAStep, bd + k * kBStep, idesc,
                              (kb > 0 || k > 0) ? 1u : 0u);
+          }
           issued = true;
           // frees this stage in both CTAs once these MMAs have read it
           umma_commit_pair(smem_addr(&empty[stage]), kBothCtas);
-          if (++stage == kSt) { stage = 0; phase ^= 1u; }
+          if (++stage == nst) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
         umma_commit_pair(smem_addr(&tfull[acc]), kBothCtas);  // accumulators ready
@@ -841,8 +850,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     }
     for (int32_t u = pair; u < wk.units; u += num_pairs, ++it) {
       const Unit t = unit_of<KIND>(wk, u);
-      const int acc = it % kBufs;
-      const uint32_t acc_phase = (uint32_t)(it / kBufs) & 1u;
+      const int acc = wide == 2 ? 0 : it & 1;
+      const uint32_t acc_phase = (uint32_t)(wide == 2 ? it : it >> 1) & 1u;
       const int64_t row0 = (int64_t)t.m_blk * kPairM + (int64_t)rank * kBM + quarter * 32;
       const RowInfo q = row_info<KIND>(p, wk, M, row0 + lane);
       const bool got = mbar_wait(smem_addr(&tfull[acc]), acc_phase, abort_flag);
@@ -853,8 +862,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       else if (KIND == GEMM_DZ) epi_dz(p, &map_c, M, t, q, row0, roff, lane, tb, st);
       else if (KIND == GEMM_DX) {
 #pragma unroll 1
-        for (int g = 0; g < kNacc; ++g)
-          epi_dx(p, &map_c, M, wk, t, q, t.n_blk * kNacc + g, row0, lane,
+        for (int g = 0; g < wide; ++g)
+          epi_dx(p, &map_c, M, wk, t, q, t.n_blk * wide + g, row0, lane,
                  tb + (uint32_t)(g * kBN), st);
       } else {
         const bool more = ahead && u + num_pairs < wk.units;

@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(kDxrThreads) k_dx_reduce(Geometry g, int32_t j
   pdl_begin();
   const int64_t M = rows_of_sample(w.err, j, KID_DX_REDUCE);
   const int64_t mb = ceil_div(M, kPairM);
-  const int S = w.err[ERR_DX_SPLITS];  // written by the dX GEMM of this sample
+  const int S = w.err[ERR_DX_SPLITS];  // the dX GEMM's plan
   if (S == 1 || M <= 0) return;
   if (S < 1 || S > kMaxSplits || S * mb > dxp_row_block_cap(g)) {  // not a count it can write
     if (blockIdx.x == 0 && threadIdx.x == 0)
@@ -548,10 +548,10 @@ __global__ void __launch_bounds__(kDxrThreads) k_dx_reduce(Geometry g, int32_t j
 }
 
 // ---------------------------------------------------------------------------
-// Xm^T [H, dz_rows] from Xm [m_pad, H] for rows [0, round_up(M, 256)) of the
-// current sample, into columns [off, off + round_up(M, 256)) with off the
-// pairing offset (0 without pairing; rows past M are the gather's zeros, so the
-// K padding of the dW GEMM reads zeros). With Xm^T the dW GEMM's B operand is
+// The backward's first kernel: Xm^T [H, dz_rows] from Xm [m_pad, H] for rows
+// [0, round_up(M, 256)) of the current sample, into columns [off, off +
+// round_up(M, 256)) with off the pairing offset (0 without pairing; rows past M
+// are the gather's zeros, so the K padding of the dW GEMM reads zeros). With Xm^T the dW GEMM's B operand is
 // K-major: one K-major and two MN-major boxes per stage instead of four
 // MN-major boxes, which measured 12% faster. A block moves a 256-row x
 // 64-column tile through shared memory with 16-byte global loads and stores,
@@ -565,7 +565,7 @@ constexpr int kTrThreads = 256;
 constexpr int kTrChunks = kTrRows * kTrCols / 8 / kTrThreads;   // 16-byte chunks per thread
 
 __global__ void __launch_bounds__(kTrThreads) k_xm_transpose(Geometry g, int32_t j, bool defer,
-                                                             WsPtrs w) {
+                                                             int num_pairs, WsPtrs w) {
   pdl_begin();
   const int32_t M = rows_of_sample(w.err, j, KID_XM_TRANSPOSE);
   if (!BGPO_IN_BOUNDS(w.err, M <= g.m_cap, KID_XM_TRANSPOSE * 16 + 9)) return;
@@ -580,6 +580,17 @@ __global__ void __launch_bounds__(kTrThreads) k_xm_transpose(Geometry g, int32_t
       w.err[ERR_PEND_OFF] = (int32_t)round_up(M, kBK);
       w.err[ERR_PEND] = pend_tag(j);
     }
+  }
+  if (blockIdx.x == gridDim.x - 1) {
+    // one more block: the plan of the dX GEMM, which took 1.1 us of that kernel's start
+    if (blockIdx.y == 0 && threadIdx.x < 32) {
+      const DxPlan plan = dx_plan_warp(g, M, num_pairs);
+      if (threadIdx.x == 0) {
+        w.err[ERR_DX_SPLITS] = plan.splits;
+        w.err[ERR_DX_WIDE] = plan.wide;
+      }
+    }
+    return;
   }
   const int64_t r0 = (int64_t)blockIdx.x * kTrRows;
   const int64_t h0 = (int64_t)blockIdx.y * kTrCols;
@@ -744,10 +755,10 @@ cudaError_t launch_dx_reduce(const Geometry& g, int32_t j, const WsPtrs& w, floa
   return launch_dependent(k_dx_reduce, (unsigned)grid, kDxrThreads, 0, s, g, j, w, dX);
 }
 
-cudaError_t launch_xm_transpose(const Geometry& g, int32_t j, bool defer, const WsPtrs& w,
-                                cudaStream_t s) {
-  const dim3 grid((unsigned)(g.m_pad / kTrRows), (unsigned)ceil_div(g.H, kTrCols));
-  return launch_dependent(k_xm_transpose, grid, kTrThreads, 0, s, g, j, defer, w);
+cudaError_t launch_xm_transpose(const Geometry& g, int32_t j, bool defer, int num_pairs,
+                                const WsPtrs& w, cudaStream_t s) {
+  const dim3 grid((unsigned)(g.m_pad / kTrRows) + 1, (unsigned)ceil_div(g.H, kTrCols));
+  return launch_dependent(k_xm_transpose, grid, kTrThreads, 0, s, g, j, defer, num_pairs, w);
 }
 
 cudaError_t launch_group_advantage(int32_t B, int32_t G, const float* rewards, float* A_out,
