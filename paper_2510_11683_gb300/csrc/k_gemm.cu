@@ -5,9 +5,10 @@
 // of the pair stages rows [128 r, 128 r + 128) of the A tile and columns
 // [128 r, 128 r + 128) of the B tile, and holds accumulator rows
 // [128 r, 128 r + 128) in its TMEM. The dX GEMM's tiles are one or two such
-// tiles side by side, sharing their A tile. Roles in each CTA (192 threads):
-//   warp 0      TMA producer: 128-byte-swizzled bf16 boxes into a 6-stage ring
-//               of 32 KB (dX at two: 4 stages of 48 KB); every copy of both CTAs completes on the even CTA's
+// tiles side by side, sharing their A tile. Roles in each CTA (224 threads):
+//   warps 0, 6  TMA producers of A and of B: 128-byte-swizzled bf16 boxes into a
+//               6-stage ring of 32 KB (dX at two accumulators: 4 stages of 48
+//               KB); every copy of both CTAs completes on the even CTA's
 //               "full" barrier, which the even CTA alone arms with both CTAs'
 //               transaction bytes (a negative transaction count in between is
 //               allowed)
@@ -52,7 +53,13 @@ namespace {
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr int32_t kStatusInvalidArg = 1;  // BGPO_ERR_INVALID_ARG
 constexpr int32_t kStatusTimeout = 8;     // BGPO_ERR_TIMEOUT
-constexpr int kThreads = 192;             // 6 warps
+constexpr int kThreads = 224;             // 7 warps
+// The B producer. One thread issuing both operands' copies was busy for 375 cycles
+// a K block (counted with clock64; a K block's MMAs take 512), more with dX's and
+// dW's 64-column boxes. From two warps: 256-wide dX tiles 720 -> 585 cycles a K
+// block (500 rows, H 512, V 38912: 35.3 -> 29.8 us), dW 1205 -> 1163 us at 1,679
+// rows of the 4096 x 126464 head, forward and dZ as before.
+constexpr int kWarpB = 6;
 constexpr uint32_t kTmemCols = 2 * kBN;   // two accumulators
 constexpr uint32_t kMnChunkBytes = 64 * 64 * 2;   // one 64 x 64 bf16 TMA box (MN-major)
 constexpr uint16_t kBothCtas = 0x3;
@@ -258,12 +265,11 @@ __device__ __forceinline__ uint32_t stage_bytes(const LoadPlan& q) {
          (uint32_t)q.b_boxes * (Majors<KIND>::b_mn ? kMnChunkBytes : kTileBBytes);
 }
 
-// Issues them for the K block that starts at element k; they complete on `cbar`,
-// the even CTA's full barrier (shared::cluster address).
+// Issue the A and the B copies of the K block that starts at element k; they
+// complete on `cbar`, the even CTA's full barrier (shared::cluster address).
 template <int KIND>
-__device__ __forceinline__ void load_stage(const LoadPlan& q, const CUtensorMap* ma,
-                                           const CUtensorMap* mb, uint32_t sa, uint32_t sb,
-                                           uint32_t cbar, int32_t k) {
+__device__ __forceinline__ void load_a(const LoadPlan& q, const CUtensorMap* ma, uint32_t sa,
+                                       uint32_t cbar, int32_t k) {
   if (!Majors<KIND>::a_mn) {
     if (q.a_boxes) tma_load_2d_pair(sa, ma, cbar, q.a_x + k, q.a_y);
   } else {
@@ -271,6 +277,11 @@ __device__ __forceinline__ void load_stage(const LoadPlan& q, const CUtensorMap*
     for (int c = 0; c < kBM / 64; ++c)
       if (c < q.a_boxes) tma_load_2d_pair(sa + c * kMnChunkBytes, ma, cbar, q.a_x + c * 64, k);
   }
+}
+
+template <int KIND>
+__device__ __forceinline__ void load_b(const LoadPlan& q, const CUtensorMap* mb, uint32_t sb,
+                                       uint32_t cbar, int32_t k) {
   if (!Majors<KIND>::b_mn) {
     if (q.b_boxes) tma_load_2d_pair(sb, mb, cbar, k, q.b_y);
   } else {
@@ -756,34 +767,41 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   uint8_t* s_a = smem;
   uint8_t* s_b = smem + nst * kTileABytes;
 
-  if (warp == 0) {
-    // ---------------- TMA producer (both CTAs) ----------------
+  if (warp == 0 || warp == kWarpB) {
+    // ---------------- TMA producers (both CTAs): A tiles, B tiles ----------------
     if (lane == 0) {
+      const bool is_a = warp == 0;
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
       bool issued = false;
-      const uint32_t sa0 = smem_addr(s_a), sb0 = smem_addr(s_b);
+      const uint32_t dst0 = smem_addr(is_a ? s_a : s_b);
+      const uint32_t step = is_a ? kTileABytes : b_bytes;
       const uint32_t full0 = smem_addr(full), empty0 = smem_addr(empty);
       const uint32_t cfull0 = map_to_cta(full0, 0);
       for (int32_t u = pair; u < wk.units && ok; u += num_pairs) {
         const Unit t = unit_of<KIND>(wk, u);
         const LoadPlan lp = load_plan<KIND>(p, wk, t, rank, roff);
-        // the even CTA arms the transaction bytes of both CTAs' copies on its
-        // full barrier; the odd CTA's copies only complete_tx on it (a
-        // per-stage remote arrive from the odd CTA halved the throughput)
+        // the even CTA's A producer arms the transaction bytes of both CTAs'
+        // copies on its full barrier; the other producers' copies only
+        // complete_tx on it (a per-stage remote arrive from the odd CTA halved the
+        // throughput)
         const uint32_t bytes =
             stage_bytes<KIND>(lp) + stage_bytes<KIND>(load_plan<KIND>(p, wk, t, peer, roff));
         for (int32_t k = t.kb0 * kBK, end = (t.kb0 + t.kb_n) * kBK; k < end; k += kBK) {
           if (!mbar_wait(empty0 + stage * 8, phase ^ 1u, abort_flag)) { ok = false; break; }
-          if (rank == 0) mbar_arrive_expect_tx(full0 + stage * 8, bytes);
-          load_stage<KIND>(lp, &map_a, &map_b, sa0 + stage * kTileABytes, sb0 + stage * b_bytes,
-                           cfull0 + stage * 8, k);
+          const uint32_t dst = dst0 + stage * step, cbar = cfull0 + stage * 8;
+          if (is_a) {
+            if (rank == 0) mbar_arrive_expect_tx(full0 + stage * 8, bytes);
+            load_a<KIND>(lp, &map_a, dst, cbar, k);
+          } else {
+            load_b<KIND>(lp, &map_b, dst, cbar, k);
+          }
           issued = true;
           if (++stage == nst) { stage = 0; phase ^= 1u; }
         }
       }
-      pdl_launch_dependents();
+      if (is_a) pdl_launch_dependents();
       if (!ok) {
         raise_abort(abort_flag, peer);
         set_device_error(err, kStatusTimeout, kernel_id<KIND>() * 16 + 2);
