@@ -269,7 +269,7 @@ struct DxPlan {
 
 // Estimated cycles of the GEMM over all chunks and of the split reduction. The
 // constants are fits to 15 shapes times 10 forced plans, measured on a GB300 at
-// about 2 GHz: a K block takes 700 cycles at one accumulator and 1,030 at two, a
+// about 2 GHz: a K block takes 590 cycles at one accumulator and 1,030 at two, a
 // launch 16,000 and 19,200 beside its K loops; at two, each further wave shows its
 // epilogue; unsplit tiles, which add into dX themselves, take 12,000 and 17,400
 // longer; partials stream at 3,100 bytes per cycle.
@@ -278,7 +278,7 @@ BGPO_HD float dx_cost(const Geometry& g, int64_t M, int num_pairs, int wide, int
       (uint32_t)(ceil_div(M, kPairM) * dx_tiles_n(g.tiles_h, wide)) * (uint32_t)s;
   const float waves = (float)((units + (uint32_t)num_pairs - 1) / (uint32_t)num_pairs);
   const float kb = (float)(((uint32_t)g.kb_vc_min + (uint32_t)s - 1) / (uint32_t)s);
-  float gemm = waves * kb * (wide == 1 ? 700.f : 1030.f);
+  float gemm = waves * kb * (wide == 1 ? 590.f : 1030.f);
   gemm += wide == 1 ? 16000.f : 9200.f + 10000.f * waves;
   if (s == 1) gemm += wide == 1 ? 12000.f : 17400.f * waves;
   // passes over M x H floats: each partial once and dX twice in the reduction, and
