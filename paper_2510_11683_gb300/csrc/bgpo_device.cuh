@@ -328,9 +328,10 @@ __device__ __forceinline__ void pdl_launch_dependents() {
 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// The head of a kernel without a prologue of its own.
-__device__ __forceinline__ void pdl_begin() {
-  pdl_launch_dependents();
+// The head of a kernel without a prologue of its own. `early`: the next kernel may
+// start at once; otherwise when this one has ended.
+__device__ __forceinline__ void pdl_begin(bool early = true) {
+  if (early) pdl_launch_dependents();
   pdl_wait();
 }
 

@@ -264,8 +264,9 @@ constexpr int kDzVec = 4;                           // 8-column vectors per thre
 constexpr int kDzItemVecs = kDzThreads * kDzVec;    // 1024 vectors = 8192 columns
 
 __global__ void __launch_bounds__(kDzThreads, 4)
-    k_dz_from_logits(Geometry g, int32_t j, int64_t chunk, const float* coef, WsPtrs w) {
-  pdl_begin();
+    k_dz_from_logits(Geometry g, int32_t j, int64_t chunk, const float* coef, bool early,
+                     WsPtrs w) {
+  pdl_begin(early);
   const int32_t M = rows_of_sample(w.err, j, KID_DZ_FROM_LOGITS);
   if (w.err[ERR_LOGITS] != 1) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -518,9 +519,9 @@ __device__ __forceinline__ void dx_reduce_row(const Geometry& g, const WsPtrs& w
   }
 }
 
-__global__ void __launch_bounds__(kDxrThreads) k_dx_reduce(Geometry g, int32_t j, WsPtrs w,
-                                                           float* dX) {
-  pdl_begin();
+__global__ void __launch_bounds__(kDxrThreads) k_dx_reduce(Geometry g, int32_t j, bool early,
+                                                           WsPtrs w, float* dX) {
+  pdl_begin(early);
   const int64_t M = rows_of_sample(w.err, j, KID_DX_REDUCE);
   const int64_t mb = ceil_div(M, kPairM);
   const int S = w.err[ERR_DX_SPLITS];  // the dX GEMM's plan
@@ -565,8 +566,9 @@ constexpr int kTrThreads = 256;
 constexpr int kTrChunks = kTrRows * kTrCols / 8 / kTrThreads;   // 16-byte chunks per thread
 
 __global__ void __launch_bounds__(kTrThreads) k_xm_transpose(Geometry g, int32_t j, bool defer,
-                                                             int num_pairs, WsPtrs w) {
-  pdl_begin();
+                                                             int num_pairs, bool early,
+                                                             WsPtrs w) {
+  pdl_begin(early);
   const int32_t M = rows_of_sample(w.err, j, KID_XM_TRANSPOSE);
   if (!BGPO_IN_BOUNDS(w.err, M <= g.m_cap, KID_XM_TRANSPOSE * 16 + 9)) return;
   const int64_t off = row_offset(w.err[ERR_ROW_OFF], w.dz_rows, g.m_pad);
@@ -672,6 +674,15 @@ __global__ void k_selftest_wait(int32_t* err, uint64_t timeout_ns) {
 
 }  // namespace
 
+// Whether the backward's small kernels let the GEMM after them start at once. A
+// GEMM block that takes an SM's shared memory leaves a kernel that streams through
+// L1 less of it: with batches of 2^23 response hidden values and more they run
+// longer than the launch they would hide. Early -> late: 8 x 512 responses on the
+// 4096 x 126464 head with kept logits 8747 -> 8651 us, 16 x 512 in chunks 21960 ->
+// 21855, 8 x 256 6043 -> 6047; below, 6 x 333 on a 1536 x 50001 head 1367 -> 1371,
+// a sample on a 2048 x 32000 one 261.6 -> 263.5, on a 1024 x 8192 one 65.8 -> 67.5.
+static bool starts_next_early(const Geometry& g) { return g.m_cap * g.H < (int64_t(1) << 23); }
+
 cudaError_t launch_selftest_wait(int32_t* err, uint64_t timeout_ns, cudaStream_t s) {
   return launch_dependent(k_selftest_wait, 1, 32, 0, s, err, timeout_ns);
 }
@@ -722,7 +733,7 @@ cudaError_t launch_dz_from_logits(const Geometry& g, int32_t j, int64_t chunk, c
   const int64_t most = g.m_pad * ceil_div(g.vc / 8, kDzItemVecs);
   const int64_t grid = most < 4 * (int64_t)num_sms ? most : 4 * (int64_t)num_sms;
   return launch_dependent(k_dz_from_logits, (unsigned)grid, kDzThreads, 0, s, g, j, chunk, coef,
-                          w);
+                          starts_next_early(g), w);
 }
 
 cudaError_t launch_seq_reduce(const Geometry& g, int32_t j, const WsPtrs& w, float* ell_out,
@@ -752,13 +763,15 @@ cudaError_t launch_dx_reduce(const Geometry& g, int32_t j, const WsPtrs& w, floa
     grid = ceil_div(g.m_cap * (g.H / 4), kDxrThreads);
     if (grid > kDxrFlatBlocks) grid = kDxrFlatBlocks;
   }
-  return launch_dependent(k_dx_reduce, (unsigned)grid, kDxrThreads, 0, s, g, j, w, dX);
+  return launch_dependent(k_dx_reduce, (unsigned)grid, kDxrThreads, 0, s, g, j,
+                          starts_next_early(g), w, dX);
 }
 
 cudaError_t launch_xm_transpose(const Geometry& g, int32_t j, bool defer, int num_pairs,
                                 const WsPtrs& w, cudaStream_t s) {
   const dim3 grid((unsigned)(g.m_pad / kTrRows) + 1, (unsigned)ceil_div(g.H, kTrCols));
-  return launch_dependent(k_xm_transpose, grid, kTrThreads, 0, s, g, j, defer, num_pairs, w);
+  return launch_dependent(k_xm_transpose, grid, kTrThreads, 0, s, g, j, defer, num_pairs,
+                          starts_next_early(g), w);
 }
 
 cudaError_t launch_group_advantage(int32_t B, int32_t G, const float* rewards, float* A_out,
