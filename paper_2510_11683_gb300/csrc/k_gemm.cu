@@ -198,14 +198,19 @@ __device__ __forceinline__ int64_t b_base(const GemmParams& p) {
   return KIND == GEMM_DZ ? p.v_begin : 0;
 }
 
-// Whether this CTA's 128 rows of a K-major A tile hold any masked row. A tile
-// past them is not loaded: the MMA multiplies what the stage happens to hold,
-// into accumulator rows that no epilogue reads. With the epilogues' row checks
-// this leaves out up to three quarters of dZ's traffic at few rows: 4096 x 126464
-// head, one response of 99 and 221 masked rows, step 2087 -> 2004 us; 2048 x 32000
-// head, 301 to 424 rows, 1125 -> 1060 us (with the split rule in integers).
-__device__ __forceinline__ bool a_has_rows(const Work& w, const Unit& t, uint32_t rank) {
-  return t.m_blk * kPairM + (int32_t)rank * kBM < w.rows;
+// Whether this CTA loads its 128 rows of a K-major A tile: when they hold a masked
+// row. A tile past them is not read by any epilogue; the MMA then multiplies what
+// the stage happens to hold. With the epilogues' row checks this leaves out up to
+// three quarters of dZ's traffic at few rows: 4096 x 126464 head, one response of
+// 99 and 221 masked rows, step 2087 -> 2004 us; 2048 x 32000 head, 301 to 424
+// rows, 1125 -> 1060 us (with the split rule in integers). From two row blocks on
+// the forward and dZ GEMMs load Xm's zero rows all the same: they are bound by
+// power, and zeros cost the multipliers less of it than stale numbers (1,124 and
+// 983 rows, forwards 1473 -> 1456 us; 568 and 1,515 rows, step 6209 -> 6170; 1,336
+// and 828 rows of a 1536 x 50001 head 1373 -> 1364).
+template <int KIND>
+__device__ __forceinline__ bool loads_a(const Work& w, const Unit& t, uint32_t rank) {
+  return t.m_blk * kPairM + (int32_t)rank * kBM < w.rows || (KIND != GEMM_DX && w.tiles_m > 1);
 }
 
 // The copies of one CTA for the stages of one unit: everything about them that
@@ -234,7 +239,7 @@ __device__ __forceinline__ LoadPlan load_plan(const GemmParams& p, const Work& w
   if (!Majors<KIND>::a_mn) {
     q.a_x = KIND == GEMM_DX ? (int32_t)p.dz_col0 : 0;
     q.a_y = a0 + (KIND == GEMM_DX ? (int32_t)roff : 0);
-    q.a_boxes = a_has_rows(w, t, rank) ? 1 : 0;
+    q.a_boxes = loads_a<KIND>(w, t, rank) ? 1 : 0;
   } else {
     // dZ^T: 2 boxes of 64 vocabulary columns x 64 masked rows, inside the dZ buffer
     q.a_x = (int32_t)(p.dz_col0 + a0);
