@@ -67,6 +67,7 @@ struct MaskArgs {
   uint8_t* mask_out;  // may be null
   const int32_t* resp_len;  // may be null: [B] real response lengths
   bool pair_dw = false;     // BGPO_FLAG_PAIR_DW: an odd sample may pair with a pending one
+  bool clear_err = false;   // clear the error word and forget a pending sample first
 };
 
 cudaError_t launch_mask_compact(const MaskArgs& a, const WsPtrs& w, cudaStream_t s);

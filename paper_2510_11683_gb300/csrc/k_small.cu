@@ -46,7 +46,13 @@ __global__ void __launch_bounds__(kScanThreads) k_mask_compact(MaskArgs a, WsPtr
   const int64_t Q = ((int64_t)a.R + 3) / 4;
   const int64_t nblk = (int64_t)a.B * Q;
   const uint64_t d_over_2_24 = (a.t_mode == 1) ? (uint64_t)a.n_t : 1ull;   // D / 2^24
-  if (tid == 0) s_carry = 0;
+  if (tid == 0) {
+    s_carry = 0;
+    if (a.clear_err) {
+      w.err[ERR_STATUS] = w.err[ERR_WHERE] = 0;
+      w.err[ERR_PEND] = -1;
+    }
+  }
   // t of every sequence: T = u24 + 1 (i.i.d.) or j 2^24 + u24 + 1 (stratified)
   for (int32_t b = tid; b < a.B; b += kScanThreads) {
     const uint64_t bg = (uint64_t)b + (uint64_t)a.b_offset;   // global sequence index
