@@ -609,15 +609,15 @@ __device__ __forceinline__ void epi_dx(const GemmParams& p, const CUtensorMap* m
 // there at up to 6.7 (plain copy: 6.4), so each warp fetches the lines of the
 // pair's next tile into L2 while it adds the current one, in halves (512-byte
 // row segments): whole tiles at once measured 5-12% slower, quarters and eighths
-// slower than no prefetch. Before -> after, in us: V 126464, H 4096: 829 -> 618
-// (31 rows), 835 -> 700 (505), 911 -> 844 (1012), 1204 -> 1045 (1521), 1470 ->
-// 1335 (2027); V 152064, H 3584: 855 -> 653 (62), 967 -> 907 (1012); V 32000,
-// H 2048: 106 -> 90 (62), 131 -> 121 (1012). From 2,500 rows on the two are within
-// the noise (1591 -> 1657, 1636 -> 1616 at 2536; 2489 -> 2568 at 4056). A dW
-// that L2 holds needs no fetching (V 8192, H 1024: 14 -> 18 at 62 rows), and row
-// segments that do not start on a 128-byte line gain nothing (V 50001, H 1032:
-// 86 -> 90 at 505 rows, 106 -> 102 at 1012).
-constexpr int64_t kDwPrefetchKb = 32;                      // K blocks: 2,048 rows
+// slower than no prefetch. Without -> with, in us: V 126464, H 4096: 829 -> 618
+// (31 rows), 835 -> 700 (505), 911 -> 844 (1012), 1204 -> 1045 (1521), 1425 ->
+// 1310 (2154), 1643 -> 1491 (2536), 1893 -> 1817 (3042), but 1901 -> 1979 (3298)
+// and 3147 -> 3278 (5073); V 152064, H 3584: 855 -> 653 (62), 967 -> 907 (1012),
+// 1547 -> 1445 (2282), 1999 -> 1963 (3042); V 32000, H 2048: 106 -> 90 (62), 131 ->
+// 121 (1012), 199 -> 189 (2282). A dW that L2 holds needs no fetching (V 8192, H
+// 1024: 14 -> 18 at 62 rows), and row segments that do not start on a 128-byte
+// line gain nothing (V 50001, H 1032: 86 -> 90 at 505 rows, 106 -> 102 at 1012).
+constexpr int64_t kDwPrefetchKb = 48;                      // K blocks: 3,072 rows
 constexpr int64_t kDwPrefetchMinBytes = int64_t(1) << 27;  // about L2's size
 
 __device__ __forceinline__ bool dw_prefetches(const GemmParams& p, const Work& w) {

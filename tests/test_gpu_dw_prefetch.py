@@ -3,7 +3,7 @@
 The smallest dW that prefetches, with a ragged last vocabulary block and a
 32-column last hidden-size tile, the same just below the size line, a hidden
 size whose rows do not start on 128-byte lines (no prefetch), and K on both
-sides of the 2,048-row line: l, dX and dW against the fp64 oracle within the tolerances of
+sides of the 3,072-row line: l, dX and dW against the fp64 oracle within the tolerances of
 the parity tests (l 1e-3 relative, gradients 2e-2 normwise).
 """
 import numpy as np
@@ -29,7 +29,8 @@ def _lib():
     (20, 2056, 16400, False),    # H % 32 != 0
     (20, 2080, 16201, True),     # K over a pending sample's rows too
     (1030, 1024, 32800, False),  # 467 and 1,616 rows
-    (1030, 1024, 32800, True),   # K = 2,128 rows: past the line
+    (1030, 1024, 32800, True),   # K = 2,128 rows
+    (1600, 1024, 32800, True),   # K over 3,072 rows: past the line
 ])
 def test_prefetching_dw_matches_the_oracle(R, H, V, pair):
     wl = Workload("dw_prefetch", B=2, P=3, R=R, H=H, V=V, n_t=2, G=2, t_mode=1, seed=21,
