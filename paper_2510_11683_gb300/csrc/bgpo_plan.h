@@ -209,7 +209,7 @@ BGPO_HD int64_t chunk_end(const Geometry& g, int64_t c) {
 struct WsLayout {
   size_t err;        // int32[16]: the fields of ErrField
   size_t t;          // float[B]    t_{b,j}
-  size_t tnum;       // uint32[2B]  T numerator (t = T / D), (low, high) words
+  size_t tnum;       // uint32[2B]  T numerator (t = T / D), (low, high) words (several mask rounds)
   size_t seg_off;    // int32[B+1]  first compacted row of each sequence
   size_t rows;       // int32[m_cap] b*R + i of each masked position, ascending
   size_t tgt;        // int32[m_pad] target token of each compacted row
