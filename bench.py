@@ -53,10 +53,10 @@ UNIT = "tokens/s"
 # workload while the GEMM sources hash to `sha`; otherwise the line reports
 # traffic as null.
 TRAFFIC = {
-    "sha": "981f980e3a7dad317219b89f4aa070d106cc6dba692a8370f6e7e2c06829d45a",
+    "sha": "46e139b2d199cb3071375714308d1caf53107ffc0fcad5e91cf3cf5a54cd2a59",
     "workload": "llada8b_r512_onpolicy",
-    "bytes_per_launch": {"lmhead_fwd_lse": 1.561e9, "lmhead_dz": 3.275e9, "dx_gemm": 4.363e9,
-                         "dw_gemm": 14.406e9},
+    "bytes_per_launch": {"lmhead_fwd_lse": 2.090e9, "lmhead_dz": 3.227e9, "dx_gemm": 4.613e9,
+                         "dw_gemm": 16.271e9},
     "source": "ncu over the 56 GEMM launches of one bench step (llada8b_r512_onpolicy, dW paired), "
               "mean per launch",
 }
