@@ -578,6 +578,8 @@ __global__ void __launch_bounds__(kDxrThreads) k_dx_reduce(Geometry g, int32_t j
                                                            WsPtrs w, float* dX) {
   pdl_begin(early);
   const int64_t M = rows_of_sample(w.err, j, KID_DX_REDUCE);
+  // the flat forms below walk as many tiles as M asks for
+  if (!BGPO_IN_BOUNDS(w.err, M <= g.m_cap, KID_DX_REDUCE * 16 + 10)) return;
   const int64_t mb = ceil_div(M, kPairM);
   const int S = w.err[ERR_DX_SPLITS];  // the dX GEMM's plan
   if (S == 1 || M <= 0) return;
