@@ -50,10 +50,12 @@
  *    launching call returns BGPO_ERR_UNSUPPORTED_DEVICE.
  *  - A checked build of the same library (compiled with -DBGPO_CHECKED) tests
  *    every index it reads from device memory (masked-row lists, segment
- *    offsets, row counts, split counts) and every target token against its
- *    buffer before use; a failed test records BGPO_ERR_BOUNDS in the error word
- *    and skips the access. It stands in for a memory checker. The normal build
- *    trusts these values, which its own kernels wrote.
+ *    offsets, row counts) and every target token against its buffer before use;
+ *    a failed test records BGPO_ERR_BOUNDS in the error word and skips the
+ *    access. It stands in for a memory checker. The normal build trusts these
+ *    values, which its own kernels wrote. Both builds test the dX plan (tile
+ *    width, split count): one that does not fit the sample records
+ *    BGPO_ERR_INVALID_ARG, and the sample's dX is added unsplit.
  */
 #ifndef BGPO_H_
 #define BGPO_H_

@@ -294,6 +294,19 @@ BGPO_HD bool dx_fits(const Geometry& g, int64_t M, const DxPlan& c) {
   return c.splits <= g.kb_vc_min && c.splits * ceil_div(M, kPairM) <= dxp_row_block_cap(g);
 }
 
+// The plan that the dX GEMM and the split reduction after it run on, from the two
+// words the backward's first kernel left. Both take it from here, so that the
+// reduction sums exactly what the GEMM stored. Words that hold no plan for this
+// sample (a damaged workspace: dx_plan always fits) make an unsplit one, which adds
+// straight into dX, and `*fits` false.
+BGPO_HD DxPlan dx_plan_stored(const Geometry& g, int64_t M, int32_t wide, int32_t splits,
+                              bool* fits) {
+  const DxPlan p = {wide, splits};
+  *fits = (wide == 1 || wide == kDxWide) && splits >= 1 && splits <= kMaxSplits &&
+          dx_fits(g, M, p);
+  return *fits ? p : DxPlan{kDxWide, 1};
+}
+
 // The plan, given the candidate of least cost (M > 0).
 BGPO_HD DxPlan dx_plan_of(const Geometry& g, int64_t M, int num_pairs, const DxPlan& best,
                           float cost) {

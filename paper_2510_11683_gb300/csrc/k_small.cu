@@ -581,13 +581,11 @@ __global__ void __launch_bounds__(kDxrThreads) k_dx_reduce(Geometry g, int32_t j
   // the flat forms below walk as many tiles as M asks for
   if (!BGPO_IN_BOUNDS(w.err, M <= g.m_cap, KID_DX_REDUCE * 16 + 10)) return;
   const int64_t mb = ceil_div(M, kPairM);
-  const int S = w.err[ERR_DX_SPLITS];  // the dX GEMM's plan
-  if (S == 1 || M <= 0) return;
-  if (S < 1 || S > kMaxSplits || S * mb > dxp_row_block_cap(g)) {  // not a count it can write
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-      set_device_error(w.err, kStatusInvalidArg, KID_DX_REDUCE * 16 + 2);
-    return;
-  }
+  if (M <= 0) return;
+  // the dX GEMM's plan (which reports one that does not fit, and runs unsplit)
+  bool fits;
+  const int S = dx_plan_stored(g, M, w.err[ERR_DX_WIDE], w.err[ERR_DX_SPLITS], &fits).splits;
+  if (S == 1) return;
   const int64_t split_stride = mb * kPairM * g.H / 4;
   const int64_t nvec = g.H / 4;
   float4* out = reinterpret_cast<float4*>(dX);
