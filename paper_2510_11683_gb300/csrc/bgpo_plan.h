@@ -267,6 +267,18 @@ struct DxPlan {
   int32_t wide, splits;
 };
 
+// K blocks of the longest of s splits, summed over the chunks: the last chunk may be
+// much narrower than the others (V 115266 in chunks of 16,384 leaves one of 578).
+// Charging every chunk the narrowest one's blocks made two splits look cheap there:
+// GEMM and reduction 338 -> 207 us at 521 rows of 528, V 55165 in chunks of 13,568
+// 566 -> 459 at 3,321 rows of 1,472, V 108141 in chunks of 15,360 337 -> 213 at 105
+// rows of 3,112.
+BGPO_HD uint32_t dx_kblocks(const Geometry& g, int s) {
+  const uint32_t n = (uint32_t)s, full = (uint32_t)(g.vc / kBK);
+  const uint32_t last = (uint32_t)ceil_div(g.V - (g.n_vc - 1) * g.vc, kBK);
+  return (uint32_t)(g.n_vc - 1) * ((full + n - 1) / n) + (last + n - 1) / n;
+}
+
 // Estimated cycles of the GEMM over all chunks and of the split reduction. The
 // constants are fits to 15 shapes times 10 forced plans, measured on a GB300 at
 // about 2 GHz: a K block takes 590 cycles at one accumulator and 1,030 at two, a
@@ -277,15 +289,14 @@ BGPO_HD float dx_cost(const Geometry& g, int64_t M, int num_pairs, int wide, int
   const uint32_t units =
       (uint32_t)(ceil_div(M, kPairM) * dx_tiles_n(g.tiles_h, wide)) * (uint32_t)s;
   const float waves = (float)((units + (uint32_t)num_pairs - 1) / (uint32_t)num_pairs);
-  const float kb = (float)(((uint32_t)g.kb_vc_min + (uint32_t)s - 1) / (uint32_t)s);
-  float gemm = waves * kb * (wide == 1 ? 590.f : 1030.f);
-  gemm += wide == 1 ? 16000.f : 9200.f + 10000.f * waves;
-  if (s == 1) gemm += wide == 1 ? 12000.f : 17400.f * waves;
+  float launch = wide == 1 ? 16000.f : 9200.f + 10000.f * waves;
+  if (s == 1) launch += wide == 1 ? 12000.f : 17400.f * waves;
+  const float kloops = waves * (float)dx_kblocks(g, s) * (wide == 1 ? 590.f : 1030.f);
   // passes over M x H floats: each partial once and dX twice in the reduction, and
   // each partial twice for every chunk that adds to it
   const float passes = (float)(s + 2 + 2 * s * (int)(g.n_vc - 1));
   const float reduce = s == 1 ? 2600.f : 4000.f + passes * (float)M * (float)g.H * (4.f / 3100.f);
-  return gemm * (float)g.n_vc + reduce;
+  return kloops + launch * (float)g.n_vc + reduce;
 }
 
 // Candidate i of the 32: a tile width and a split count the split buffer has room for.
