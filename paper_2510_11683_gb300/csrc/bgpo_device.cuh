@@ -345,14 +345,15 @@ __device__ __forceinline__ void pdl_begin(bool early = true) {
 __device__ __forceinline__ DxPlan dx_plan_warp(const Geometry& g, int32_t M, int num_pairs) {
   static_assert(2 * kMaxSplits == 32, "one candidate per lane");
   if (M <= 0) return DxPlan{kDxWide, 1};
+  const DxPlan usual = dx_plan_usual(g, M, num_pairs);
   const DxPlan c = dx_candidate((int)(threadIdx.x & 31));
   // costs are positive: their bits order as they do
-  const uint32_t cost = dx_fits(g, M, c)
+  const uint32_t cost = dx_allowed(g, M, usual, c)
                             ? __float_as_uint(dx_cost(g, M, num_pairs, c.wide, c.splits))
                             : 0xffffffffu;
   const uint32_t least = __reduce_min_sync(0xffffffffu, cost);
   const int who = __ffs(__ballot_sync(0xffffffffu, cost == least)) - 1;
-  return dx_plan_of(g, M, num_pairs, dx_candidate(who), __uint_as_float(least));
+  return dx_plan_of(g, M, num_pairs, usual, dx_candidate(who), __uint_as_float(least));
 }
 
 // ---- misc -----------------------------------------------------------------------

@@ -249,20 +249,16 @@ BGPO_HD int64_t dxp_row_block_cap(const Geometry& g) {
 }
 
 // Tile width and split count of the dX GEMM of a sample with M masked rows (the
-// same for every chunk of the sample): 256 x 512 tiles split by dx_splits, unless
-// another pair of the two is estimated to take at least 5% less (dx_cost). That is
-// so where a split's K loop is short against its epilogue and its partials, and
-// where H leaves a second accumulator empty. GEMM and reduction, 512-wide tiles
-// -> now, in us: M 291, H 152, V 137580: 153 -> 113; M 4398, H 104, V 84350: 247 ->
-// 183; M 300, H 1024, V 8192: 22.1 -> 17.4; M 5331, H 2712, V 975 (split twice ->
-// unsplit): 116 -> 62; M 110, H 808, V 14743 in chunks of 1,024: 185 -> 132. Over
-// 36 shapes drawn from H 64 .. 4096, V 512 .. 152,064, 1 .. 16,384 response rows
-// the geometric mean is 1.22 times faster and none is slower by more than 1%. Over
-// vocabulary chunks, where every split's partial is read and written again for
-// each chunk, fewer splits win (against the time of the same sample's dZ GEMM,
-// which the power cap slows alike): H 3584, V 152064, 5 chunks: 1.29 times faster
-// at 1,259 rows (13 -> 2 splits), 1.11 at 4,893, 1.02 at 10,165, 0.99 at 12,489;
-// H 4096, V 126464, 4 chunks: 1.04 at 951 rows, 1.06 at 2,027, 1.03 at 4,286.
+// same for every chunk of the sample): 256 x 512 tiles split by dx_splits (the usual
+// plan), unless another allowed pair of the two (dx_allowed) is estimated to take at
+// least 5% less (dx_cost). That is so where a split's K loop is short against its
+// epilogue and its partials, and where H leaves a second accumulator empty. GEMM and
+// reduction, usual plan -> now, in us: M 283, H 152, V 137580: 152 -> 83; M 4429, H
+// 104, V 84350: 221 -> 176; M 309, H 1024, V 8192: 23.4 -> 17.2; M 5281, H 2712, V 975
+// (3 splits -> unsplit): 119 -> 66; M 107, H 808, V 14743 in chunks of 1,024: 185 ->
+// 131; M 521, H 528, V 115266 in chunks of 16,384: 352 -> 166. Over 36 shapes drawn
+// from H 64 .. 4096, V 512 .. 152,064, 1 .. 16,384 response rows the geometric mean is
+// 1.26 times faster and none is slower by more than 1%.
 struct DxPlan {
   int32_t wide, splits;
 };
@@ -318,25 +314,51 @@ BGPO_HD DxPlan dx_plan_stored(const Geometry& g, int64_t M, int32_t wide, int32_
   return *fits ? p : DxPlan{kDxWide, 1};
 }
 
-// The plan, given the candidate of least cost (M > 0).
-BGPO_HD DxPlan dx_plan_of(const Geometry& g, int64_t M, int num_pairs, const DxPlan& best,
-                          float cost) {
-  const DxPlan usual = {kDxWide, dx_splits(ceil_div(M, kPairM), dx_tiles_n(g.tiles_h), num_pairs,
-                                           g.kb_vc_min, dxp_row_block_cap(g))};
+// The usual plan of M > 0 rows.
+BGPO_HD DxPlan dx_plan_usual(const Geometry& g, int64_t M, int num_pairs) {
+  return DxPlan{kDxWide, dx_splits(ceil_div(M, kPairM), dx_tiles_n(g.tiles_h), num_pairs,
+                                   g.kb_vc_min, dxp_row_block_cap(g))};
+}
+
+// Most K blocks that one accumulator adds up in a plan of s splits.
+BGPO_HD int64_t dx_chain(const Geometry& g, int s) {
+  return ceil_div(ceil_div(g.vc < g.V ? g.vc : g.V, kBK), s);
+}
+
+// Whether candidate c may take the usual plan's place: not with fewer splits, unless
+// the chains stay within kDxShortChain K blocks. The rounding error of an fp32
+// accumulator grows with its chain: dX against the 64-bit product of the same bf16
+// dZ and W, H 3584, V 152064, 5 chunks: 2.8e-6 with 13 splits, 6.4e-6 with 6, 1.9e-5
+// with 2, 3.6e-5 unsplit. Beside the 1-2e-3 that dZ's rounding to bf16 makes, chains
+// of up to 476 blocks moved dX's whole error by -0.1 to +0.4%; over 48 shapes with
+// chains of up to 16 blocks instead of 1 to 10 it moved by 6e-6 of itself in the mean
+// (-1.5e-4 to 2.0e-4, larger in 24 of them).
+// What fewer splits would give otherwise: H 3584, V 152064, 5 chunks: 1182 -> 897 us at
+// 1,259 rows, 3826 -> 3401 at 4,893; H 4096, V 126464, 4 chunks: 703 -> 691 at 951
+// rows, 2906 -> 2841 at 4,286.
+constexpr int64_t kDxShortChain = 16;
+BGPO_HD bool dx_allowed(const Geometry& g, int64_t M, const DxPlan& usual, const DxPlan& c) {
+  return dx_fits(g, M, c) && (c.splits >= usual.splits || dx_chain(g, c.splits) <= kDxShortChain);
+}
+
+// The plan, given the allowed candidate of least cost.
+BGPO_HD DxPlan dx_plan_of(const Geometry& g, int64_t M, int num_pairs, const DxPlan& usual,
+                          const DxPlan& best, float cost) {
   return cost <= 0.95f * dx_cost(g, M, num_pairs, usual.wide, usual.splits) ? best : usual;
 }
 
 BGPO_HD DxPlan dx_plan(const Geometry& g, int64_t M, int num_pairs) {
   if (M <= 0) return DxPlan{kDxWide, 1};
-  DxPlan best = dx_candidate(0);   // one split always fits
+  const DxPlan usual = dx_plan_usual(g, M, num_pairs);
+  DxPlan best = usual;   // always a candidate
   float cost = dx_cost(g, M, num_pairs, best.wide, best.splits);
-  for (int i = 1; i < 2 * kMaxSplits; ++i) {
+  for (int i = 0; i < 2 * kMaxSplits; ++i) {
     const DxPlan c = dx_candidate(i);
-    if (!dx_fits(g, M, c)) continue;
+    if (!dx_allowed(g, M, usual, c)) continue;
     const float t = dx_cost(g, M, num_pairs, c.wide, c.splits);
     if (t < cost) { cost = t; best = c; }
   }
-  return dx_plan_of(g, M, num_pairs, best, cost);
+  return dx_plan_of(g, M, num_pairs, usual, best, cost);
 }
 
 // `keep_logits` appends the fp32 logit region. `pair_dw` doubles the rows of
