@@ -104,6 +104,9 @@ def _ptr(t, dtype=None, name="tensor", cur=None):
     if (isinstance(t, _TORCH.Tensor) and t.is_cuda and t.get_device() == cur
             and (dtype is None or t.dtype is dtype) and t.is_contiguous()):
         return t.data_ptr()
+    if cur < 0 and isinstance(t, _TORCH.Tensor) and t.is_cuda:
+        # a tensor that native code made before torch.cuda was initialised
+        return _ptr(t, dtype, name, _TORCH.cuda.current_device())
     _refuse(t, dtype, name)
 
 
@@ -125,8 +128,8 @@ def _refuse(t, dtype, name):
 
 
 def _current_device():
-    """Index of the current CUDA device, or -1 while CUDA is not initialised (no tensor
-    is on the GPU then, and _ptr refuses every tensor)."""
+    """Index of the current CUDA device, or -1 while torch.cuda is not initialised (a
+    tensor is then on the GPU only where native code put it there: _ptr asks again)."""
     torch = _torch()
     return torch._C._cuda_getDevice() if torch.cuda.is_initialized() else -1
 
