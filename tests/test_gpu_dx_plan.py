@@ -2,7 +2,14 @@
 several vocabulary chunks, ragged hidden sizes and last row blocks. dX against
 the fp64 oracle (2e-2 normwise, the parity tests' tolerance), rows no sample
 masked exactly zero, and the same bits from a second run.
+
+The plan that the device's warp form leaves in the workspace is compared with the
+host's sequential one (csrc/bgpo_plan.h), kind by kind.
 """
+import os
+import shutil
+import subprocess
+
 import numpy as np
 import pytest
 
@@ -13,9 +20,9 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("B,R,H,V,chunk", [
-    (1, 300, 1032, 900, 0),      # 256-wide, few splits
-    (2, 700, 2712, 500, 0),      # 256-wide, unsplit
-    (2, 700, 2712, 1300, 512),   # unsplit or split, added over three chunks
+    (1, 300, 1032, 900, 0),      # short K, split
+    (2, 700, 2712, 500, 0),      # 8 K blocks, unsplit
+    (2, 700, 2712, 1300, 512),   # added over three chunks, the last narrower
     (1, 40, 104, 9000, 0),       # one column block, 16 splits
     (1, 40, 808, 3000, 1024),    # split, three chunks
     (4, 600, 200, 3000, 0),      # many row blocks, one column block
@@ -38,3 +45,82 @@ def test_dx_plans_match_the_oracle(B, R, H, V, chunk):
     assert normwise(got, o["dX"]) <= 2e-2
     assert not got[~o["masks"].any(axis=0).astype(bool)].any()
     assert torch.equal(a["dX"], b["dX"]) and torch.equal(a["dW"], b["dW"])
+
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_2510_11683_gb300", "csrc")
+
+# lines "rows H V chunk pair M pairs wide splits" -> the host's plan, its estimate and
+# that of the plan given
+HOST_PLAN = r"""
+#include <cstdio>
+#include "bgpo_plan.h"
+using namespace bgpo;
+int main() {
+  long long rows, H, V, chunk, pair, M, pairs, wide, splits;
+  while (std::scanf("%lld %lld %lld %lld %lld %lld %lld %lld %lld", &rows, &H, &V, &chunk, &pair,
+                    &M, &pairs, &wide, &splits) == 9) {
+    const Geometry g = make_geometry(1, 0, rows, H, V, chunk, pair != 0);
+    const DxPlan p = dx_plan(g, M, (int)pairs), u = dx_plan_usual(g, M, (int)pairs);
+    std::printf("%d %d %.9g %.9g %.9g\n", p.wide, p.splits,
+                dx_cost(g, M, (int)pairs, p.wide, p.splits),
+                dx_cost(g, M, (int)pairs, (int)wide, (int)splits),
+                dx_cost(g, M, (int)pairs, u.wide, u.splits));
+  }
+}
+"""
+
+
+def test_the_devices_plan_is_the_hosts(tmp_path):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    gxx = shutil.which("g++")
+    if gxx is None:
+        pytest.skip("no g++")
+    ensure_built()
+    import paper_2510_11683_gb300 as bg
+    pairs = torch.cuda.get_device_properties(0).multi_processor_count // 2
+    lines, got = [], []
+    for R, H, V, chunk, pair in [
+            (300, 1032, 900, 0, False), (1400, 2712, 500, 0, False), (1400, 2712, 1300, 512, False),
+            (40, 104, 9000, 0, False), (40, 808, 3000, 1024, False), (2400, 200, 3000, 0, False),
+            (600, 4096, 700, 0, False), (780, 2056, 6000, 0, False), (3, 64, 65, 0, False),
+            (1000, 528, 20000, 4096, False), (5000, 4096, 2000, 0, False),
+            (9728, 2048, 20000, 0, False), (9728, 512, 5000, 1280, True),
+            (4864, 4096, 6000, 4864, False)]:
+        # stratified over 8 samples: from an eighth of the rows to all of them
+        prob = bg.problem(1, 0, R, H, V, 8, 1, t_mode=bg.T_STRATIFIED, seed=R + H,
+                          vocab_chunk=chunk, pair_dw=pair)
+        ws = bg.alloc_workspace(prob)
+        X = torch.randn((1, R, H), device="cuda").to(torch.bfloat16)
+        W = (torch.randn((V, H), device="cuda") * H ** -0.5).to(torch.bfloat16)
+        Y = torch.randint(0, V, (1, R), dtype=torch.int32, device="cuda")
+        ell, coef = torch.empty(1, device="cuda"), torch.ones(1, device="cuda")
+        dX, dW = torch.zeros((1, R, H), device="cuda"), torch.zeros((V, H), device="cuda")
+        for j in range(8):
+            bg.sample_mask(prob, j, ws)
+            bg.elbo_fwd(prob, j, X, W, Y, ws, ell)
+            bg.elbo_bwd_accumulate(prob, j, X, W, Y, coef, ws, dX, dW)
+            word = ws[:64].view(torch.int32).tolist()
+            M, splits, wide = word[3], word[5], word[11]
+            assert word[0] == 0
+            if M:
+                lines.append(f"{R} {H} {V} {chunk} {int(pair)} {M} {pairs} {wide} {splits}")
+                got.append((wide, splits))
+    src, exe = tmp_path / "plan.cpp", tmp_path / "plan"
+    src.write_text(HOST_PLAN)
+    subprocess.run([gxx, "-std=c++17", "-O1", f"-I{CSRC}", str(src), "-o", str(exe)], check=True)
+    out = subprocess.run([str(exe)], input="\n".join(lines), check=True, capture_output=True,
+                         text=True).stdout.split("\n")
+    assert len(got) > 100
+    for line, (wide, splits), host in zip(lines, got, out):
+        p_wide, p_splits, best, mine, usual = host.split()
+        if (wide, splits) != (int(p_wide), int(p_splits)):
+            # the two compilers contract multiplies and adds differently: a tie, or a
+            # gain on the 5% line, may fall either way
+            best, mine, usual = float(best), float(mine), float(usual)
+            near = min(abs(mine - best), abs(mine - 0.95 * usual), abs(best - 0.95 * usual))
+            assert near <= 1e-5 * best, (line, host)
+    kinds = {(wide, splits > 1) for wide, splits in got}
+    assert kinds == {(1, False), (1, True), (2, False), (2, True)}, kinds
