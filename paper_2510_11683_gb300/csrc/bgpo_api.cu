@@ -1,7 +1,8 @@
 // Host side of the C ABI declared in include/bgpo.h: argument validation,
 // workspace layout, TMA tensor-map encoding, kernel launches, per-kernel
-// event tracing and an NVTX range named after each launching call. Keeps no state between calls except the cached driver entry
-// point of cuTensorMapEncodeTiled.
+// event tracing and an NVTX range named after each launching call. Keeps no state
+// between calls except the cached driver entry point of cuTensorMapEncodeTiled and
+// each device's SM count (g_sms).
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <math.h>

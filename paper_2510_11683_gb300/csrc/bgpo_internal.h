@@ -14,8 +14,8 @@ namespace bgpo {
 // be written while its blocks already exist, so they are not read through the
 // read-only path (no __ldg, no const __restrict__ on them). A sample is 9 to 12
 // launches of 2 to 5 us around its GEMMs: launching and draining them in turn
-// cost 33 us of a 5-kernel forward (1024 x 8192 head; 25 us now) and 80 of the
-// 1205 us of a 4-sample step on a 32,000 x 2048 head.
+// made a 5-kernel forward of 25 us (1024 x 8192 head; 19 us by now) one of 33, and cost
+// 80 of the 1205 us of a 4-sample step on a 32,000 x 2048 head.
 template <class... Params, class... Args>
 cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem,
                              cudaStream_t s, Args... args) {

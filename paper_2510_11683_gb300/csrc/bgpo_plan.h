@@ -122,8 +122,8 @@ BGPO_HD void row_group_tile(int64_t u, int64_t tiles_m, int64_t tiles_n, int64_t
 // wave-quantised time ceil(tiles*s/pairs)/s is within 8% of the ideal
 // tiles/pairs, else the best s. s * mb never exceeds `row_block_cap`, which
 // bounds the partial buffer independently of the SM count.
-// Integers only: every thread of the GEMM runs this, and 16 rounds of 64-bit and
-// double-precision divisions took 3 us of its start.
+// Integers only: every lane of the warp that makes the plan runs this, at the start of
+// the backward, and 16 rounds of 64-bit and double-precision divisions took 3 us.
 BGPO_HD int dx_splits(int64_t mb, int64_t tiles_n, int num_pairs, int64_t k_blocks,
                       int64_t row_block_cap) {
   if (mb * tiles_n <= 0 || num_pairs <= 0) return 1;
@@ -347,6 +347,8 @@ BGPO_HD DxPlan dx_plan_of(const Geometry& g, int64_t M, int num_pairs, const DxP
   return cost <= 0.95f * dx_cost(g, M, num_pairs, usual.wide, usual.splits) ? best : usual;
 }
 
+// The rule one candidate after the other. The device takes dx_plan_warp, one candidate
+// per lane; tests hold that against this.
 BGPO_HD DxPlan dx_plan(const Geometry& g, int64_t M, int num_pairs) {
   if (M <= 0) return DxPlan{kDxWide, 1};
   const DxPlan usual = dx_plan_usual(g, M, num_pairs);

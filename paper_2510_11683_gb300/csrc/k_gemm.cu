@@ -617,8 +617,11 @@ __device__ __forceinline__ void epi_dx(const GemmParams& p, const CUtensorMap* m
 // and 3147 -> 3278 (5073); V 152064, H 3584: 855 -> 653 (62), 967 -> 907 (1012),
 // 1547 -> 1445 (2282), 1999 -> 1963 (3042); V 32000, H 2048: 106 -> 90 (62), 131 ->
 // 121 (1012), 199 -> 189 (2282). A dW that L2 holds needs no fetching (V 8192, H
-// 1024: 14 -> 18 at 62 rows), and row segments that do not start on a 128-byte
-// line gain nothing (V 50001, H 1032: 86 -> 90 at 505 rows, 106 -> 102 at 1012).
+// 1024: 14 -> 18 at 62 rows), and a hidden size that is no multiple of 32 gained
+// nothing (V 50001, H 1032: 86 -> 90 at 505 rows, 106 -> 102 at 1012). Where dW starts
+// does not matter: 16 bytes off a 128-byte line the 4096 x 126464 head takes 901 -> 635
+// at 30 rows, 938 -> 705 at 498, 1290 -> 1095 at 1,507, 1852 -> 1637 at 2,512 (on the
+// line 799 -> 608, 827 -> 676, 1205 -> 1032, 1705 -> 1551).
 constexpr int64_t kDwPrefetchKb = 48;                      // K blocks: 3,072 rows
 constexpr int64_t kDwPrefetchMinBytes = int64_t(1) << 27;  // about L2's size
 

@@ -731,11 +731,14 @@ __global__ void k_selftest_wait(int32_t* err, uint64_t timeout_ns) {
 
 // Whether the backward's small kernels let the GEMM after them start at once. A
 // GEMM block that takes an SM's shared memory leaves a kernel that streams through
-// L1 less of it: with batches of 2^23 response hidden values and more they run
-// longer than the launch they would hide. Early -> late: 8 x 512 responses on the
-// 4096 x 126464 head with kept logits 8747 -> 8651 us, 16 x 512 in chunks 21960 ->
-// 21855, 8 x 256 6043 -> 6047; below, 6 x 333 on a 1536 x 50001 head 1367 -> 1371,
-// a sample on a 2048 x 32000 one 261.6 -> 263.5, on a 1024 x 8192 one 65.8 -> 67.5.
+// L1 less of it: large batches may then run longer than the launch they would hide.
+// Early -> late: 8 x 512 responses on the 4096 x 126464 head with kept logits 8747 ->
+// 8651 us, 16 x 512 in chunks 21960 -> 21855, 8 x 256 6043 -> 6047; 6 x 333 on a 1536
+// x 50001 head 1367 -> 1371, a sample on a 2048 x 32000 one 261.6 -> 263.5, on a 1024 x
+// 8192 one 65.8 -> 67.5. The line at 2^23 response hidden values lies between those
+// cases but is not an optimum: at ten sizes from 2^21 to 2^25 either choice is within
+// the spread with the default flags (early / late 0.97-1.01), and with kept logits late
+// is 0-4% faster at all of them, also below the line.
 static bool starts_next_early(const Geometry& g) { return g.m_cap * g.H < (int64_t(1) << 23); }
 
 cudaError_t launch_selftest_wait(int32_t* err, uint64_t timeout_ns, cudaStream_t s) {
