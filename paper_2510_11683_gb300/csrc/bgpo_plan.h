@@ -321,8 +321,9 @@ BGPO_HD DxPlan dx_plan_usual(const Geometry& g, int64_t M, int num_pairs) {
 }
 
 // Most K blocks that one accumulator adds up in a plan of s splits.
-BGPO_HD int64_t dx_chain(const Geometry& g, int s) {
-  return ceil_div(ceil_div(g.vc < g.V ? g.vc : g.V, kBK), s);
+BGPO_HD uint32_t dx_chain(const Geometry& g, int s) {
+  const uint32_t kb = (uint32_t)ceil_div(g.vc < g.V ? g.vc : g.V, kBK);
+  return (kb + (uint32_t)s - 1) / (uint32_t)s;
 }
 
 // Whether candidate c may take the usual plan's place: not with fewer splits, unless
@@ -336,7 +337,7 @@ BGPO_HD int64_t dx_chain(const Geometry& g, int s) {
 // What fewer splits would give otherwise: H 3584, V 152064, 5 chunks: 1182 -> 897 us at
 // 1,259 rows, 3826 -> 3401 at 4,893; H 4096, V 126464, 4 chunks: 703 -> 691 at 951
 // rows, 2906 -> 2841 at 4,286.
-constexpr int64_t kDxShortChain = 16;
+constexpr uint32_t kDxShortChain = 16;
 BGPO_HD bool dx_allowed(const Geometry& g, int64_t M, const DxPlan& usual, const DxPlan& c) {
   return dx_fits(g, M, c) && (c.splits >= usual.splits || dx_chain(g, c.splits) <= kDxShortChain);
 }

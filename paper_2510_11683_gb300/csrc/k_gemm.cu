@@ -85,7 +85,6 @@ struct Work {
   int32_t splits;
   int32_t wide;      // accumulators per tile (dX: one or two)
   int32_t rows;      // A rows that hold data: CTAs and warps wholly past them skip theirs
-  bool planned;      // dX: the error word holds a plan that fits
 };
 
 struct Unit {
@@ -104,7 +103,6 @@ __device__ __forceinline__ Work make_work(const GemmParams& p, int32_t M, int64_
   w.kb_first = 0;
   w.groups = 1;
   w.rows = M;
-  w.planned = true;
   if (KIND == GEMM_FWD || KIND == GEMM_DZ) {
     w.tiles_m = (int32_t)ceil_div(M, kPairM);
     w.tiles_n = (int32_t)(KIND == GEMM_FWD ? p.g.n_vt : ceil_div(p.v_end - p.v_begin, kBN));
@@ -117,8 +115,11 @@ __device__ __forceinline__ Work make_work(const GemmParams& p, int32_t M, int64_
     w.kb_total = (int32_t)ceil_div(p.v_end - p.v_begin, kBK);
     // one plan for every chunk of the sample (the partials of split s
     // accumulate over the chunks), left by the kernel that transposed Xm
+    bool fits;
     const DxPlan plan =
-        dx_plan_stored(p.g, M, p.w.err[ERR_DX_WIDE], p.w.err[ERR_DX_SPLITS], &w.planned);
+        dx_plan_stored(p.g, M, p.w.err[ERR_DX_WIDE], p.w.err[ERR_DX_SPLITS], &fits);
+    if (!fits && M > 0 && blockIdx.x == 0 && threadIdx.x == 0)
+      set_device_error(p.w.err, kStatusInvalidArg, KID_DX_GEMM * 16 + 6);
     w.wide = plan.wide;
     w.splits = plan.splits;
     w.tiles_n = (int32_t)dx_tiles_n(p.g.tiles_h, w.wide);
@@ -770,8 +771,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       set_device_error(err, kStatusInvalidArg, kernel_id<KIND>() * 16 + 5);
     err[ERR_PEND] = -1;  // nothing waits any more
   }
-  if (KIND == GEMM_DX && M > 0 && !wk.planned && blockIdx.x == 0 && threadIdx.x == 0)
-    set_device_error(err, kStatusInvalidArg, kernel_id<KIND>() * 16 + 6);
   // tiles of two accumulators fill TMEM (one tile at a time) and take 48 KB a stage
   const int wide = KIND == GEMM_DX ? wk.wide : 1;
   const int nst = wide == 2 ? kDxStages : kStages;
