@@ -301,18 +301,17 @@ BGPO_HD bool dx_fits(const Geometry& g, int64_t M, const DxPlan& c) {
   return c.splits <= g.kb_vc_min && c.splits * ceil_div(M, kPairM) <= dxp_row_block_cap(g);
 }
 
-// The plan that the dX GEMM and the split reduction after it run on, from the two
-// words the backward's first kernel left. Both take it from here, so that the
-// reduction sums exactly what the GEMM stored. Words that hold no plan for this
-// sample (a damaged workspace: dx_plan always fits) make an unsplit one, which adds
-// straight into dX, and `*fits` false.
-BGPO_HD DxPlan dx_plan_stored(const Geometry& g, int64_t M, int32_t wide, int32_t splits,
-                              bool* fits) {
-  const DxPlan p = {wide, splits};
-  *fits = (wide == 1 || wide == kDxWide) && splits >= 1 && splits <= kMaxSplits &&
-          dx_fits(g, M, p);
-  return *fits ? p : DxPlan{kDxWide, 1};
+// The split count that the dX GEMM and the split reduction after it run with, from the
+// word the backward's first kernel left. Both take it from here, so that the reduction
+// sums exactly what the GEMM stored. A word that holds no count for this sample (a
+// damaged workspace: dx_plan always fits) makes an unsplit GEMM, which adds straight
+// into dX, and `*fits` false. (Any tile width the other word may hold is one of the two
+// that work: dx_wide_stored. The reduction need not know it.)
+BGPO_HD int dx_splits_stored(const Geometry& g, int64_t M, int32_t splits, bool* fits) {
+  *fits = splits >= 1 && splits <= kMaxSplits && dx_fits(g, M, DxPlan{kDxWide, splits});
+  return *fits ? splits : 1;
 }
+BGPO_HD int dx_wide_stored(int32_t wide) { return wide == 1 ? 1 : kDxWide; }
 
 // The usual plan of M > 0 rows.
 BGPO_HD DxPlan dx_plan_usual(const Geometry& g, int64_t M, int num_pairs) {

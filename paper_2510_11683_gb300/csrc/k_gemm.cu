@@ -116,12 +116,10 @@ __device__ __forceinline__ Work make_work(const GemmParams& p, int32_t M, int64_
     // one plan for every chunk of the sample (the partials of split s
     // accumulate over the chunks), left by the kernel that transposed Xm
     bool fits;
-    const DxPlan plan =
-        dx_plan_stored(p.g, M, p.w.err[ERR_DX_WIDE], p.w.err[ERR_DX_SPLITS], &fits);
+    w.splits = dx_splits_stored(p.g, M, p.w.err[ERR_DX_SPLITS], &fits);
+    w.wide = dx_wide_stored(p.w.err[ERR_DX_WIDE]);
     if (!fits && M > 0 && blockIdx.x == 0 && threadIdx.x == 0)
       set_device_error(p.w.err, kStatusInvalidArg, KID_DX_GEMM * 16 + 6);
-    w.wide = plan.wide;
-    w.splits = plan.splits;
     w.tiles_n = (int32_t)dx_tiles_n(p.g.tiles_h, w.wide);
     w.units = w.tiles_m * w.tiles_n * w.splits;
   } else {  // GEMM_DW

@@ -577,18 +577,14 @@ __device__ __forceinline__ void dx_reduce_row(const Geometry& g, const WsPtrs& w
 __global__ void __launch_bounds__(kDxrThreads) k_dx_reduce(Geometry g, int32_t j, bool early,
                                                            WsPtrs w, float* dX) {
   pdl_begin(early);
-  // read beside the row count: after its test the kernel takes 10.08 us at 495 rows of
-  // 1,536, so 9.86
-  const int32_t wide = w.err[ERR_DX_WIDE], splits = w.err[ERR_DX_SPLITS];
   const int64_t M = rows_of_sample(w.err, j, KID_DX_REDUCE);
   // the flat forms below walk as many tiles as M asks for
   if (!BGPO_IN_BOUNDS(w.err, M <= g.m_cap, KID_DX_REDUCE * 16 + 10)) return;
   const int64_t mb = ceil_div(M, kPairM);
-  if (M <= 0) return;
-  // the dX GEMM's plan (which reports one that does not fit, and runs unsplit)
+  // the dX GEMM's count (which reports one that does not fit, and runs unsplit)
   bool fits;
-  const int S = dx_plan_stored(g, M, wide, splits, &fits).splits;
-  if (S == 1) return;
+  const int S = dx_splits_stored(g, M, w.err[ERR_DX_SPLITS], &fits);
+  if (S == 1 || M <= 0) return;
   const int64_t split_stride = mb * kPairM * g.H / 4;
   const int64_t nvec = g.H / 4;
   float4* out = reinterpret_cast<float4*>(dX);

@@ -1,8 +1,8 @@
 """The dX plan as the GEMM and the split reduction read it back (csrc/bgpo_plan.h,
-dx_plan_stored, which both call): a plan that dx_plan makes comes back as it is;
-any other pair of words that does not fit the sample (too many splits for the
-narrowest chunk's K blocks or for the split buffer, a tile width that does not
-exist) is an unsplit plan for both, and reported.
+dx_splits_stored, which both call, and dx_wide_stored): a plan that dx_plan makes
+comes back as it is; a split count that does not fit the sample (too many for the
+narrowest chunk's K blocks or for the split buffer) is one split for both, and
+reported; a tile width that does not exist is one that does.
 """
 import os
 import shutil
@@ -29,20 +29,18 @@ int main() {
           for (int64_t M : {int64_t(1), rows}) {
             const DxPlan p = dx_plan(g, M, 76);
             bool fits = false;
-            const DxPlan q = dx_plan_stored(g, M, p.wide, p.splits, &fits);
-            bad += !fits || q.wide != p.wide || q.splits != p.splits;
+            bad += dx_splits_stored(g, M, p.splits, &fits) != p.splits || !fits;
+            bad += dx_wide_stored(p.wide) != p.wide;
             for (int32_t wide : {-1, 0, 1, 2, 3, 0x5EED0000})
-              for (int32_t s : {-0x7fffffff, -1, 0, 1, 2, 3, 5, 9, 15, 16, 17, 0x7fffffff}) {
-                const DxPlan r = dx_plan_stored(g, M, wide, s, &fits);
-                const bool ok = (wide == 1 || wide == 2) && s >= 1 && s <= kMaxSplits &&
-                                s <= g.kb_vc_min && s * ceil_div(M, kPairM) <= cap;
-                bad += ok != fits;
-                bad += ok ? (r.wide != wide || r.splits != s) : r.splits != 1;
-                bad += r.wide != 1 && r.wide != 2;
-                good += ok;
-                refused += !ok;
-                kblocks += s >= 1 && s <= kMaxSplits && s > g.kb_vc_min;
-              }
+              bad += dx_wide_stored(wide) != (wide == 1 ? 1 : 2);
+            for (int32_t s : {-0x7fffffff, -1, 0, 1, 2, 3, 5, 9, 15, 16, 17, 0x7fffffff}) {
+              const bool ok = s >= 1 && s <= kMaxSplits && s <= g.kb_vc_min &&
+                              s * ceil_div(M, kPairM) <= cap;
+              bad += dx_splits_stored(g, M, s, &fits) != (ok ? s : 1) || fits != ok;
+              good += ok;
+              refused += !ok;
+              kblocks += s >= 1 && s <= kMaxSplits && s > g.kb_vc_min;
+            }
           }
         }
   std::printf("%ld %ld %ld %ld\n", bad, good, refused, kblocks);
@@ -66,4 +64,5 @@ def test_the_gemm_and_the_reduction_read_one_plan(tmp_path):
         with open(os.path.join(CSRC, name)) as f:
             text = f.read()
         reads = [ln for ln in text.splitlines() if "err[ERR_DX_" in ln and "] = " not in ln]
-        assert len(reads) == 1 and "dx_plan_stored" in text, (name, reads)
+        assert sum("ERR_DX_SPLITS" in ln for ln in reads) == 1, (name, reads)
+        assert all("dx_splits_stored(" in ln or "dx_wide_stored(" in ln for ln in reads), reads
