@@ -53,10 +53,10 @@ UNIT = "tokens/s"
 # workload while the GEMM sources hash to `sha`; otherwise the line reports
 # traffic as null.
 TRAFFIC = {
-    "sha": "46e139b2d199cb3071375714308d1caf53107ffc0fcad5e91cf3cf5a54cd2a59",
+    "sha": "5f0f69d56ab0d3f042f72514fe8e47786928fdf3bd11c72a7f31e02f189aef57",
     "workload": "llada8b_r512_onpolicy",
-    "bytes_per_launch": {"lmhead_fwd_lse": 2.090e9, "lmhead_dz": 3.227e9, "dx_gemm": 4.613e9,
-                         "dw_gemm": 16.271e9},
+    "bytes_per_launch": {"lmhead_fwd_lse": 2.336e9, "lmhead_dz": 3.582e9, "dx_gemm": 5.384e9,
+                         "dw_gemm": 18.602e9},
     "source": "ncu over the 56 GEMM launches of one bench step (llada8b_r512_onpolicy, dW paired), "
               "mean per launch",
 }
